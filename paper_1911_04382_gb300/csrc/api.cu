@@ -275,9 +275,10 @@ void user_tree(grass_ctx_t ctx, const GraphData &g, const int64_t *eids, uint8_t
 grass_tree_t build_tree_impl(grass_ctx_t ctx, const grass_csr_t *A,
                              const std::vector<int64_t> &voff, const std::vector<int32_t> &roots,
                              const int64_t *user_eids = nullptr, const uint64_t *lsst_seed = nullptr,
-                             LsstStats *lsst_stats = nullptr) {
+                             LsstStats *lsst_stats = nullptr, bool batch = false) {
     auto *T = new grass_tree_s();
     T->ctx = ctx;
+    T->batch = batch;
     T->nroots = (int64_t)roots.size();
     T->roots_h = roots;
     T->ground = roots[0];
@@ -450,6 +451,9 @@ grass_status grass_ctx_set_param(grass_ctx_t ctx, const char *name, int64_t valu
 grass_status grass_tree_schedule_info(grass_tree_t T, int64_t *eliminated, int64_t *receivers,
                                       int64_t *contributions, int64_t cap) {
     if (!T || cap < 0) return GRASS_ERR_INVALID;
+    grass_ctx_t ctx = T->ctx;
+    API_BEGIN(ctx)
+    tree_rounds(ctx, T);
     const TreeSchedule &S = T->sched;
     for (int k = 0; k < S.rounds && k < cap; ++k) {
         if (eliminated) eliminated[k] = S.elim_off[k + 1] - S.elim_off[k];
@@ -467,7 +471,7 @@ grass_status grass_tree_schedule_info(grass_tree_t T, int64_t *eliminated, int64
         for (int k = 0; k < S.rounds && k < cap; ++k)
             contributions[k] = beg[S.rcv_off[k + 1]] - beg[S.rcv_off[k]];
     }
-    return GRASS_OK;
+    API_END
 }
 
 grass_status grass_kernel_timing_enable(grass_ctx_t ctx, int family) {
@@ -598,7 +602,7 @@ grass_status grass_build_forest(grass_ctx_t ctx, const grass_csr_t *A, int64_t n
         need(voff[k + 1] - voff[k] >= 2, "every graph of the batch needs at least 2 vertices");
         roots[k] = (int32_t)voff[k];
     }
-    *out = build_tree_impl(ctx, A, voff, roots);
+    *out = build_tree_impl(ctx, A, voff, roots, nullptr, nullptr, nullptr, true);
     API_END
 }
 
@@ -622,8 +626,12 @@ grass_status grass_tree_info(grass_tree_t T, int64_t *n, int64_t *m, int64_t *ro
     if (!T) return GRASS_ERR_INVALID;
     if (n) *n = T->g.n;
     if (m) *m = T->g.m;
-    if (rounds) *rounds = T->sched.rounds;
-    return GRASS_OK;
+    if (!rounds) return GRASS_OK;
+    grass_ctx_t ctx = T->ctx;
+    API_BEGIN(ctx)
+    tree_rounds(ctx, T);
+    *rounds = T->sched.rounds;
+    API_END
 }
 
 grass_status grass_tree_graph(grass_ctx_t ctx, grass_tree_t T, int32_t *eu, int32_t *ev,
@@ -656,9 +664,8 @@ grass_status grass_tree_solve(grass_ctx_t ctx, grass_tree_t T, int with_D, int r
     need_prec(prec);
     need(r_supported(r), "r must be 1, 2, 4, 8, 16, 24 or 32");
     if (with_D) ensure_sdd(ctx, T);
-    if (X != B) copy_d(ctx, X, B, T->g.n * r * esize(prec));
     clear_timeout(ctx);
-    tree_solve_inplace(ctx, T, with_D ? T->sdd : T->lap, r, prec, X, nullptr);
+    tree_solve_inplace(ctx, T, with_D ? T->sdd : T->lap, r, prec, X, nullptr, B);
     check_timeout(ctx);
     API_END
 }

@@ -72,10 +72,11 @@ struct ASpan {
     size_t n = 0;
 };
 
-// Bump allocation from device chunks of at least 64 MB, freed together: one
-// cudaMalloc per chunk instead of one per array (and no synchronising
-// cudaFree per array).  reset() reuses the chunks from the start.
+// Bump allocation from device chunks of at least chunk_min bytes, freed
+// together: one cudaMalloc per chunk instead of one per array (and no
+// synchronising cudaFree per array).  reset() reuses the chunks from the start.
 struct Arena {
+    size_t chunk_min = (size_t)64 << 20;
     std::vector<std::unique_ptr<DBuf<char>>> chunks;
     size_t cur = 0, off = 0;
     void reset() { cur = off = 0; }
@@ -93,7 +94,7 @@ struct Arena {
         }
         if (cur == chunks.size()) {
             auto c = std::make_unique<DBuf<char>>();
-            c->alloc(bytes > ((size_t)64 << 20) ? bytes : ((size_t)64 << 20));
+            c->alloc(bytes > chunk_min ? bytes : chunk_min);
             chunks.push_back(std::move(c));
             off = 0;
         }
@@ -359,6 +360,46 @@ struct alignas(32) Dbl4 {
     double x, y, z, w;
 };
 
+// Unit form of a single tree's solve (units.cuh, units.cu): one level per
+// grid phase, the units of a level eliminated block by block.
+constexpr int kUnitMin = 256;       // smallest unit of a level with several units
+constexpr int kUnitMax = 2048;      // largest: 16 FP32 columns of it fit shared memory
+constexpr int kUnitTop = 3584;      // largest last level (one unit, few columns a block)
+constexpr int kUnitRounds = 62;     // block-local elimination rounds (about 14 needed)
+constexpr int kUnitLevels = 5;
+// a unit's list arrays: 2B entries and two more, in whole 16-byte pieces
+__host__ __device__ inline int unit_stride(int B) { return (2 * B + 2 + 7) & ~7; }
+struct UnitLevel {
+    int64_t n = 0, nexp = 0;
+    int B = 0, nu = 0;
+    int local = 0, elim = 0;        // the most local indices / eliminated vertices of a unit
+    int32_t *ord = nullptr;         // [n] unit order -> vertex id (level 0) or index at this level
+    int32_t *lidx = nullptr;        // [n] unit order -> index at this level
+    uint32_t *nn = nullptr;         // [n] neighbours at elimination, local: n1 | n2 << 16
+    int4 *meta = nullptr;           // [nu] {eliminated, local indices, rounds | long lists << 16, first export}
+    uint16_t *roff = nullptr, *cbeg = nullptr, *clist = nullptr, *cpos = nullptr;
+    int32_t *ecore = nullptr;       // [nexp] next level's index of every export
+    int32_t *epos = nullptr, *edst = nullptr;   // [nexp] its position there, its row in exp
+    int32_t *sptr = nullptr;        // [n + 1] previous level's export rows by position
+    char *exp = nullptr, *V = nullptr;   // scratch: exports, level vector (32 FP64 columns)
+    double *dexp = nullptr, *w = nullptr;   // factor: load exports, weights to the parent
+};
+struct UnitTree {
+    bool built = false;
+    Arena arena;
+    double *w0 = nullptr;           // [n] level 0's weights to the parent, by position
+    std::vector<UnitLevel> lv;
+};
+struct UnitFactor {
+    Arena arena;
+    std::vector<Dbl4 *> c64;        // per level, by position {1/d, w1/d, w2/d, neighbours}
+    std::vector<float4 *> c32;
+    std::vector<double *> m64;      // per level, multipliers in clist's order
+    std::vector<float *> m32;
+    double *rinv64 = nullptr;
+    float *rinv32 = nullptr;
+};
+
 // Elimination schedule of the spanning tree by rake (degree 1) and compress
 // (degree 2) rounds; numeric factors for L_T (lap) and L_T + D (sdd).
 struct TreeFactor {
@@ -371,6 +412,7 @@ struct TreeFactor {
     DBuf<float2> fm32;
     DBuf<Dbl4> bc64;                  // [n - nroots] {1/d, w1/d, w2/d, 0} by elimination position
     DBuf<float4> bc32;
+    UnitFactor unit;                  // of the unit form, when the tree has one
 };
 
 struct TreeSchedule {
@@ -410,6 +452,7 @@ struct EulerTour {
     bool built = false;
     int64_t L = 0;                   // 2 (n - nroots) positions
     DBuf<int32_t> tour, ein, eout;
+    DBuf<int32_t> par;               // [n] parent (roots: not set)
     DBuf<uint8_t> head;              // [L] 1 at each tree's first position
     DBuf<double> pw;
     DBuf<double> ipw;                // [n] 1 / pw (roots: 1)
@@ -465,12 +508,14 @@ struct grass_tree_s {
     // one root (grounded row) per graph: a spanning tree, or a spanning
     // forest with one tree per graph of a batch
     int64_t nroots = 1;
+    bool batch = false;                // from grass_build_forest: a graph alone solves as in any batch
     std::vector<int32_t> roots_h;
     grass::DBuf<int32_t> roots;        // [nroots]
     grass::DBuf<uint8_t> isroot;       // [n]
     grass::GraphData g;
     grass::DBuf<uint8_t> in_tree;     // [m]
-    grass::TreeSchedule sched;
+    grass::TreeSchedule sched;         // elimination rounds (built on demand when units.built)
+    grass::UnitTree units;             // unit form of the solve (one tree, with a tour)
     grass::EulerTour euler;
     grass::TreeFactor lap;            // L_T grounded at rho
     grass::TreeFactor sdd;            // L_T + D
@@ -552,11 +597,26 @@ void tree_schedule(grass_ctx_t ctx, grass_tree_t T);
 // every slot in tsrc; L slots), before the contraction rounds modify it.
 void euler_build(grass_ctx_t ctx, grass_tree_t T, const int32_t *tptr, const int32_t *tocc,
                  const int32_t *tsrc, int64_t L);
+// The elimination rounds of a tree that has the unit form (their sizes are
+// reported by the API; its solves do not use them).
+void tree_rounds(grass_ctx_t ctx, grass_tree_t T);
 void tree_factor(grass_ctx_t ctx, grass_tree_t T, bool with_D, TreeFactor &f);
-// In-place tree solve of the n x r block Y (prec); optionally tracks the
-// max |x| bit pattern into maxbits (device, uint64 for both precisions).
+// Algorithmic bytes of one tree solve of r columns of s bytes.
+double tree_solve_bytes(const grass_tree_s *T, int r, double s);
+
+// ---------------------------------------------------------------- units.cu
+
+// Builds U for T's tree; false when the tree keeps the elimination rounds.
+bool unit_build(grass_ctx_t ctx, grass_tree_t T, UnitTree &U);
+// Coefficients of L_T (D null) or L_T + D.
+void unit_factor(grass_ctx_t ctx, grass_tree_t T, const UnitTree &U, const double *D,
+                 UnitFactor &f);
+// In-place tree solve of the n x r block Y (prec), or from B into Y;
+// optionally tracks the max |x| bit pattern into maxbits (device, uint64 for
+// both precisions).
 void tree_solve_inplace(grass_ctx_t ctx, grass_tree_t T, const TreeFactor &f, int r,
-                        grass_prec prec, void *Y, unsigned long long *maxbits);
+                        grass_prec prec, void *Y, unsigned long long *maxbits,
+                        const void *B = nullptr);
 
 // Y = scale * (L X + Dopt .* X) over an adjacency (ptr, col, w).  scale may
 // come from a device max-bits word (pow2 rescale) when scale_from != nullptr.

@@ -86,7 +86,7 @@ __global__ void k_eu_jump(int64_t L, const int32_t *nx_in, const int32_t *d_in, 
 __global__ void k_eu_final(int64_t mt, const int32_t *es, const int32_t *owner, const int32_t *tocc,
                            const int32_t *tsrc, const int32_t *dist, const int32_t *seg_of,
                            const int64_t *voff, const double *ew, int32_t *tour, int32_t *ein,
-                           int32_t *eout, double *pw) {
+                           int32_t *eout, int32_t *par, double *pw) {
     int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= mt) return;
     const int32_t s0 = es[2 * t], s1 = es[2 * t + 1];
@@ -106,6 +106,7 @@ __global__ void k_eu_final(int64_t mt, const int32_t *es, const int32_t *owner, 
     const int64_t pin = p0 < p1 ? p0 : p1, pout = p0 < p1 ? p1 : p0;
     ein[child] = (int32_t)pin;
     eout[child] = (int32_t)pout;
+    par[child] = p0 < p1 ? u : v;
     tour[pin] = child;
     tour[pout] = -(child + 1);
     pw[child] = ew[tsrc[s0]];
@@ -219,12 +220,13 @@ void euler_build(grass_ctx_t ctx, grass_tree_t T, const int32_t *tptr, const int
     E.tour.alloc(L);
     E.ein.alloc(n);
     E.eout.alloc(n);
+    E.par.alloc(n);
     E.pw.alloc(n);
     launch(ctx, k_eu_final, cdiv(mt, kBlock), kBlock, 0, mt, (const int32_t *)es.p,
            (const int32_t *)owner.p, tocc, tsrc, (const int32_t *)d0.p,
            g.nseg > 1 ? (const int32_t *)g.seg_of.p : nullptr,
            g.nseg > 1 ? (const int64_t *)g.seg_voff_d.p : nullptr, (const double *)g.ew64.p,
-           E.tour.p, E.ein.p, E.eout.p, E.pw.p);
+           E.tour.p, E.ein.p, E.eout.p, E.par.p, E.pw.p);
     E.head.alloc(L);
     memset_d(ctx, E.head.p, 0, L);
     launch(ctx, k_eu_roots, cdiv(T->nroots, kBlock), kBlock, 0, T->nroots,

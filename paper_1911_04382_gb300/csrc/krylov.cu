@@ -267,7 +267,7 @@ __device__ inline void grid_cols2(const double *part0, double *s_out0, const dou
 // a caller with the same mapping
 // reads X at once.  preset: the caller has already set X = 0, R = Z = Y and
 // passed a grid barrier since.
-template <typename T, int R, bool EU = false>
+template <typename T, int R, bool EU, bool UNITS>
 __device__ __forceinline__ bool cg_dev(const CGArgs<T> &g, const TreeKArgs<T> &tk,
                                        unsigned int &epoch, T *ys, bool preset = false) {
     static_assert(!EU || R == 1, "the scan-form solve handles one column");
@@ -342,7 +342,7 @@ __device__ __forceinline__ bool cg_dev(const CGArgs<T> &g, const TreeKArgs<T> &t
         if constexpr (EU) {
             if (!euler_solve_dev<T, true>(g.eu, g.Z, tk.bar, tk.budget, tk.err, epoch, mx)) return false;
         } else {
-            if (!tree_solve_dev<T, R, false>(tk, g.Z, epoch, mx, ys)) return false;
+            if (!tree_solve_dev<T, R, false, UNITS>(tk, g.Z, epoch, mx, ys)) return false;
             if (!grid_sync(tk.bar, tk.budget, tk.err, epoch)) return false;
         }
 #pragma unroll
@@ -626,13 +626,13 @@ __device__ __forceinline__ bool cg_dev(const CGArgs<T> &g, const TreeKArgs<T> &t
     return true;
 }
 
-template <typename T, int R, bool EU>
+template <typename T, int R, bool EU, bool UNITS>
 __global__ void __launch_bounds__(cg_max_threads<R, EU>(), 1)
     k_cg_persist(CGArgs<T> g, TreeKArgs<T> tk) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned int epoch = 0;
     if constexpr (!EU) tree_tail_stage<T, R>(tk, reinterpret_cast<T *>(smem_raw));
-    cg_dev<T, R, EU>(g, tk, epoch, reinterpret_cast<T *>(smem_raw));
+    cg_dev<T, R, EU, UNITS>(g, tk, epoch, reinterpret_cast<T *>(smem_raw));
 }
 
 // S's adjacency in the tree's preorder numbering (row k = the row of vertex
@@ -732,10 +732,10 @@ static void cg_persistent(grass_ctx_t ctx, grass_sparsifier_t S, bool with_D, co
     }
     const int threads = bounded_threads(
         ctx->tree_threads, eu ? cg_max_threads<R, (R == 1)>() : cg_max_threads<R, false>());
-    const void *kern = eu ? (const void *)k_cg_persist<T, R, (R == 1)>
-                          : (const void *)k_cg_persist<T, R, false>;
-    const int grid = eu ? coop_grid(ctx, k_cg_persist<T, R, (R == 1)>, threads, smem, n * Lay<R>::TPR)
-                        : coop_grid(ctx, k_cg_persist<T, R, false>, threads, smem, n * Lay<R>::TPR);
+    const auto kern = eu ? k_cg_persist<T, R, (R == 1), false>
+                     : Tr->units.built ? k_cg_persist<T, R, false, true>
+                                       : k_cg_persist<T, R, false, false>;
+    const int grid = coop_grid(ctx, kern, threads, smem, n * Lay<R>::TPR);
     if ((size_t)grid * 32 * 2 > ctx->partials.n) fail(GRASS_ERR_CUDA, "partials buffer too small");
     // the chunked element loops (one FP32 column) take 16-byte accesses;
     // all their vectors are the context's own scratch (Y is gathered by
@@ -752,10 +752,8 @@ static void cg_persistent(grass_ctx_t ctx, grass_sparsifier_t S, bool with_D, co
     // X, R, Z written (12 nrs; the first iteration's P = Z copies, 2 nrs
     // less); the start Y read and X, R, Z written (4 nrs); the end max |X|
     // (nrs) and, in preorder, the scatter of X (2 nrs)
-    const TreeSchedule &TS = Tr->sched;
     const double s = (double)sizeof(T), nrs = (double)n * R * s;
-    const double tree_b = 4.0 * nrs + TS.n_rcv * (16.0 + 2.0 * s) +
-                          (n - (double)Tr->nroots) * (16.0 + 4.0 * s);
+    const double tree_b = tree_solve_bytes(Tr, R, s);
     const double spmv_b = 4.0 * (n + 1) + S->s_nnz * (4.0 + s) + 2.0 * nrs + (with_D ? n * s : 0.0);
     const bool timing = ctx->tfam == GRASS_KF_CG;
     size_t snap = ctx->iter_launches.size();
@@ -766,7 +764,8 @@ static void cg_persistent(grass_ctx_t ctx, grass_sparsifier_t S, bool with_D, co
     }
     bool timed = ctx->t_begin(GRASS_KF_CG, 0.0);
     void *args[] = {&a, &tk};
-    GCK(cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(threads), args, smem, ctx->stream));
+    GCK(cudaLaunchCooperativeKernel((const void *)kern, dim3(grid), dim3(threads), args, smem,
+                                    ctx->stream));
     ctx->launches++;
     ctx->t_end(timed);
     if (timing) ctx->t_snap(a.iter_acc, snap, 1);
@@ -825,8 +824,7 @@ int64_t s_solve(grass_ctx_t ctx, grass_sparsifier_t S, bool with_D, int r, grass
     const size_t es = esize(prec);
     const TreeFactor &f = with_D ? T->sdd : T->lap;
     if (S->is_tree) {
-        copy_d(ctx, X, Y, total * es);
-        tree_solve_inplace(ctx, T, f, r, prec, X, maxbits);
+        tree_solve_inplace(ctx, T, f, r, prec, X, maxbits, Y);
         return 0;
     }
     if (ctx->lmax_amg && !with_D && r == 1) {
@@ -963,7 +961,7 @@ struct PCGArgs {
     double *out;                  // [0] += iterations, [1] = final r.r
 };
 
-template <typename T, int MODE>
+template <typename T, int MODE, bool UNITS>
 __global__ void __launch_bounds__(kFusedMaxThreads, 1)
     k_pcg_persist(PCGArgs<T> a, CGArgs<T> in, TreeKArgs<T> tk) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1009,7 +1007,7 @@ __global__ void __launch_bounds__(kFusedMaxThreads, 1)
         double rz = 0.0, rr = 0.0, aprev = 0.0;
         int k = 0, steps = 0;
         for (bool first = true;; first = false) {
-            if (!tree_solve_dev<T, 1, false>(tk, zc, epoch, mx, ys)) return;
+            if (!tree_solve_dev<T, 1, false, UNITS>(tk, zc, epoch, mx, ys)) return;
             if (!grid_sync(tk.bar, tk.budget, tk.err, epoch)) return;
             Acc<T> aq, arz, ax;
             for (int64_t i0 = gt; i0 < a.n; i0 += 2 * nth) {
@@ -1147,10 +1145,10 @@ __global__ void __launch_bounds__(kFusedMaxThreads, 1)
         // the inner CG leaves every z[i] written by the thread that reads it
         // below; the tree solve writes out of order and needs the barrier
         if constexpr ((MODE == 1)) {
-            if (!tree_solve_dev<T, 1, false>(tk, a.z, epoch, mx, ys)) return;
+            if (!tree_solve_dev<T, 1, false, UNITS>(tk, a.z, epoch, mx, ys)) return;
             if (!grid_sync(tk.bar, tk.budget, tk.err, epoch)) return;
         } else {
-            if (!cg_dev<T, 1>(in, tk, epoch, ys, true)) return;
+            if (!cg_dev<T, 1, false, UNITS>(in, tk, epoch, ys, true)) return;
         }
         // first: rz = r.z, rr = r.r;  later: r.z and r.z_old for beta
         acc0[0] = acc1[0] = Acc<T>();
@@ -1278,12 +1276,11 @@ static int pcg_fused(grass_ctx_t ctx, grass_sparsifier_t S, const T *rhs, T *e, 
     // 1: the tree solve alone; 2: one inner CG step on the sparsifier, in
     // closed form; 0: the inner CG as a device function
     const int mode = (S->is_tree || inner_maxit <= 0) ? 1 : (inner_maxit == 1 ? 2 : 0);
-    const void *kern = mode == 1 ? (const void *)k_pcg_persist<T, 1>
-                     : mode == 2 ? (const void *)k_pcg_persist<T, 2>
-                                 : (const void *)k_pcg_persist<T, 0>;
-    const int grid = mode == 1 ? coop_grid(ctx, k_pcg_persist<T, 1>, threads, smem, n)
-                   : mode == 2 ? coop_grid(ctx, k_pcg_persist<T, 2>, threads, smem, n)
-                               : coop_grid(ctx, k_pcg_persist<T, 0>, threads, smem, n);
+    const bool un = Tr->units.built;
+    const auto kern = mode == 1   ? (un ? k_pcg_persist<T, 1, true> : k_pcg_persist<T, 1, false>)
+                      : mode == 2 ? (un ? k_pcg_persist<T, 2, true> : k_pcg_persist<T, 2, false>)
+                                  : (un ? k_pcg_persist<T, 0, true> : k_pcg_persist<T, 0, false>);
+    const int grid = coop_grid(ctx, kern, threads, smem, n);
     PCGArgs<T> a;
     a.n = n;
     a.aptr = g.adj_ptr.p;
@@ -1345,10 +1342,8 @@ static int pcg_fused(grass_ctx_t ctx, grass_sparsifier_t S, const T *rhs, T *e, 
     //  mode 0: outer dots r, z, z_old; p: z, p, p; update: e, p, r, q, z read,
     //          e, r, z_old, z, R, Z written -> 17 ns, less 2 ns for the inner
     //          CG's first iteration; inner: tree_b, SpMV with S, 12 ns.
-    const TreeSchedule &TS = Tr->sched;
     const double s = (double)sizeof(T), ns = (double)n * s;
-    const double tree_b = 4.0 * ns + TS.n_rcv * (16.0 + 2.0 * s) +
-                          (n - (double)Tr->nroots) * (16.0 + 4.0 * s);
+    const double tree_b = tree_solve_bytes(Tr, 1, s);
     const double spmv_a = 4.0 * (n + 1) + 2.0 * g.m * (4.0 + s) + 3.0 * ns;
     const double csr_s = 4.0 * (n + 1) + S->s_nnz * (4.0 + s);
     double per_outer, per_inner = 0.0, start;
@@ -1373,7 +1368,8 @@ static int pcg_fused(grass_ctx_t ctx, grass_sparsifier_t S, const T *rhs, T *e, 
     }
     bool timed = ctx->t_begin(GRASS_KF_PCG, 0.0);
     void *args[] = {&a, &in, &tk};
-    GCK(cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(threads), args, smem, ctx->stream));
+    GCK(cudaLaunchCooperativeKernel((const void *)kern, dim3(grid), dim3(threads), args, smem,
+                                    ctx->stream));
     ctx->launches++;
     ctx->t_end(timed);
     if (timing) {

@@ -71,14 +71,14 @@ unsigned int *scratch_address() {
     return g_addr.back().second;
 }
 
-template <typename T, int R>
+template <typename T, int R, bool UNITS>
 __global__ void __launch_bounds__(kPersistMaxThreads, 1)
     k_tree_noalloc(TreeKArgs<T> a, T *Y) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned int epoch = 0;
     double mx = 0.0;
     tree_tail_stage<T, R>(a, reinterpret_cast<T *>(smem_raw));
-    tree_solve_dev<T, R>(a, Y, epoch, mx, reinterpret_cast<T *>(smem_raw));
+    tree_solve_dev<T, R, false, UNITS>(a, Y, epoch, mx, reinterpret_cast<T *>(smem_raw));
 }
 
 struct NoallocCall {
@@ -101,13 +101,13 @@ void launch_noalloc(const NoallocCall &c) {
     TreeKArgs<T> ka = tree_kargs<T, R>(ctx, c.T, *c.f, &smem);
     ka.bar = c.scratch;
     ka.err = reinterpret_cast<int *>(c.scratch + 8);
-    const int grid = coop_grid(ctx, k_tree_noalloc<T, R>, ctx->tree_threads, smem,
-                               c.T->g.n * Lay<R>::TPR);
-    if ((int64_t)grid * (2 * (int64_t)ka.rounds + 2) >= kMaxArrivals)
+    const auto kern = c.T->units.built ? k_tree_noalloc<T, R, true> : k_tree_noalloc<T, R, false>;
+    const int grid = coop_grid(ctx, kern, ctx->tree_threads, smem, c.T->g.n * Lay<R>::TPR);
+    if ((int64_t)grid * (2 * (int64_t)std::max(ka.rounds, ka.u.nl) + 2) >= kMaxArrivals)
         fail(GRASS_ERR_INVALID, "tree schedule too long for the no-allocation barrier counter");
     T *Y = static_cast<T *>(c.Y);
     void *args[] = {&ka, &Y};
-    GCK(cudaLaunchCooperativeKernel((const void *)k_tree_noalloc<T, R>, dim3(grid),
+    GCK(cudaLaunchCooperativeKernel((const void *)kern, dim3(grid),
                                     dim3(ctx->tree_threads), args, smem, ctx->stream));
     ctx->launches++;
 }

@@ -13,9 +13,24 @@ __global__ void __launch_bounds__(kPersistMaxThreads, 1)
     unsigned int epoch = 0;
     double mx = 0.0;
     tree_tail_stage<T, R>(a, reinterpret_cast<T *>(smem_raw));
-    if (!tree_solve_dev<T, R>(a, Y, epoch, mx, reinterpret_cast<T *>(smem_raw))) return;
+    if (!tree_solve_dev<T, R, true, false>(a, Y, epoch, mx, reinterpret_cast<T *>(smem_raw))) return;
     if (maxbits) block_atomic_max(maxbits, mx);
 }
+
+// unit form (units.cuh), from B into Y
+template <typename T, int R>
+__global__ void __launch_bounds__(kPersistMaxThreads, 1)
+    k_tree_units(UnitArgs<T> u, unsigned int *bar, long long budget, int *err, const T *B, T *Y,
+                 unsigned long long *maxbits) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    unsigned int epoch = 0;
+    double mx = 0.0;
+    if (!unit_solve_dev<T, R, true>(u, bar, budget, err, B, Y, epoch, mx,
+                                    reinterpret_cast<T *>(smem_raw)))
+        return;
+    if (maxbits) block_atomic_max(maxbits, mx);
+}
+
 
 // scan form: grounded solve of L_T alone, one column
 template <typename T>
@@ -84,15 +99,21 @@ static void solve_rounds(grass_ctx_t ctx, grass_tree_t Tr, const TreeKArgs<T> &a
 
 template <typename T, int R>
 static void solve_T(grass_ctx_t ctx, grass_tree_t Tr, const TreeFactor &f, T *Y,
-                    unsigned long long *maxbits) {
+                    unsigned long long *maxbits, const T *B) {
     size_t smem = 0;
+    const bool scan = R == 1 && &f == &Tr->lap && ctx->euler_solve && Tr->euler.built;
+    // the unit form reads B itself; the others solve in place
+    if (B && (scan || !Tr->units.built)) {
+        copy_d(ctx, Y, B, (size_t)Tr->g.n * R * sizeof(T));
+        B = nullptr;
+    }
     TreeKArgs<T> a = tree_kargs<T, R>(ctx, Tr, f, &smem);
     if (ctx->num_sms <= 0) {
         solve_rounds<T, R>(ctx, Tr, a, Y, maxbits);
         return;
     }
     const int threads = ctx->tree_threads;
-    if (R == 1 && &f == &Tr->lap && ctx->euler_solve && Tr->euler.built) {
+    if (scan) {
         const int grid = coop_grid(ctx, k_euler_persist<T>, threads, 0, Tr->g.n);
         EulerKArgs e;
         euler_kargs<T>(ctx, Tr, grid, &e);
@@ -100,6 +121,16 @@ static void solve_T(grass_ctx_t ctx, grass_tree_t Tr, const TreeFactor &f, T *Y,
         void *eargs[] = {&e, &a, &Y, &maxbits};
         GCK(cudaLaunchCooperativeKernel((const void *)k_euler_persist<T>, dim3(grid),
                                         dim3(threads), eargs, 0, ctx->stream));
+        ctx->launches++;
+        return;
+    }
+    if (Tr->units.built) {
+        const int grid = coop_grid(ctx, k_tree_units<T, R>, threads, smem, Tr->g.n * Lay<R>::TPR);
+        GCK(cudaMemsetAsync(a.bar, 0, sizeof(unsigned int), ctx->stream));
+        if (!B) B = Y;
+        void *uargs[] = {&a.u, &a.bar, &a.budget, &a.err, &B, &Y, &maxbits};
+        GCK(cudaLaunchCooperativeKernel((const void *)k_tree_units<T, R>, dim3(grid), dim3(threads),
+                                        uargs, smem, ctx->stream));
         ctx->launches++;
         return;
     }
@@ -118,22 +149,21 @@ struct SolveCall {
     void *Y;
     unsigned long long *maxbits;
     grass_prec prec;
+    const void *B;
 };
 
 template <int R>
 static void solve_R(const SolveCall &c) {
-    if (c.prec == GRASS_FP64) solve_T<double, R>(c.ctx, c.T, *c.f, (double *)c.Y, c.maxbits);
-    else solve_T<float, R>(c.ctx, c.T, *c.f, (float *)c.Y, c.maxbits);
+    if (c.prec == GRASS_FP64) solve_T<double, R>(c.ctx, c.T, *c.f, (double *)c.Y, c.maxbits, (const double *)c.B);
+    else solve_T<float, R>(c.ctx, c.T, *c.f, (float *)c.Y, c.maxbits, (const float *)c.B);
 }
 
 void tree_solve_inplace(grass_ctx_t ctx, grass_tree_t T, const TreeFactor &f, int r,
-                        grass_prec prec, void *Y, unsigned long long *maxbits) {
-    const TreeSchedule &S = T->sched;
-    const double s = prec == GRASS_FP64 ? 8.0 : 4.0, n = (double)T->g.n;
-    const double bytes = 4.0 * n * r * s + S.n_rcv * (16.0 + 2.0 * s) +
-                         (n - (double)T->nroots) * (16.0 + 4.0 * s);
-    bool timed = ctx->t_begin(GRASS_KF_TREE, bytes);
-    SolveCall c{ctx, T, &f, Y, maxbits, prec};
+                        grass_prec prec, void *Y, unsigned long long *maxbits, const void *B) {
+    if (B == Y) B = nullptr;
+    bool timed = ctx->t_begin(GRASS_KF_TREE,
+                              tree_solve_bytes(T, r, prec == GRASS_FP64 ? 8.0 : 4.0));
+    SolveCall c{ctx, T, &f, Y, maxbits, prec, B};
     GRASS_DISPATCH_R(r, solve_R, c);
     ctx->t_end(timed);
 }

@@ -296,7 +296,8 @@ static void tree_pack(grass_ctx_t ctx, grass_tree_t T) {
     ctx->sync();
 }
 
-void tree_schedule(grass_ctx_t ctx, grass_tree_t T) {
+// rounds: build the elimination rounds even when the tree has the unit form
+static void schedule(grass_ctx_t ctx, grass_tree_t T, bool rounds) {
     const GraphData &g = T->g;
     const int64_t n = g.n;
     TreeSchedule &S = T->sched;
@@ -318,7 +319,8 @@ void tree_schedule(grass_ctx_t ctx, grass_tree_t T) {
            (const uint8_t *)T->in_tree.p, (const int64_t *)off.p, tptr.p, tocc.p, tsrc.p);
     // the scan form pays off while its FP64 tour arrays stay near the L2
     // size; larger trees keep the elimination rounds only
-    if (n <= ctx->euler_max_n) euler_build(ctx, T, tptr.p, tocc.p, tsrc.p, tslots);
+    if (n <= ctx->euler_max_n && !T->euler.built) euler_build(ctx, T, tptr.p, tocc.p, tsrc.p, tslots);
+    if (!rounds && unit_build(ctx, T, T->units)) return;
     elim_round.alloc(n);
     cls.alloc(n);
     val.alloc(n + 1);
@@ -382,6 +384,21 @@ void tree_schedule(grass_ctx_t ctx, grass_tree_t T) {
     S.d_offs.alloc(h.size());
     h2d(ctx, S.d_offs.p, h.data(), h.size() * sizeof(int64_t));
     tree_pack(ctx, T);
+}
+
+void tree_schedule(grass_ctx_t ctx, grass_tree_t T) { schedule(ctx, T, false); }
+
+void tree_rounds(grass_ctx_t ctx, grass_tree_t T) {
+    if (T->sched.rounds == 0) schedule(ctx, T, true);
+}
+
+double tree_solve_bytes(const grass_tree_s *T, int r, double s) {
+    const double n = (double)T->g.n;
+    // unit form: the vector read and written, the order, the coefficients,
+    // the list starts and the two list entries of every vertex
+    if (T->units.built) return 2.0 * n * r * s + n * (4.0 + 4.0 * s + 2.0 + 4.0);
+    return 4.0 * n * r * s + T->sched.n_rcv * (16.0 + 2.0 * s) +
+           (n - (double)T->nroots) * (16.0 + 4.0 * s);
 }
 
 // ---------------------------------------------------------------- numeric factorization
@@ -470,6 +487,10 @@ void tree_factor(grass_ctx_t ctx, grass_tree_t T, bool with_D, TreeFactor &f) {
     const GraphData &g = T->g;
     const TreeSchedule &S = T->sched;
     const int64_t n = g.n;
+    if (T->units.built) {
+        unit_factor(ctx, T, T->units, with_D ? g.D64.p : nullptr, f.unit);
+        return;
+    }
     f.invd64.alloc(n);
     f.b1_64.alloc(n);
     f.b2_64.alloc(n);

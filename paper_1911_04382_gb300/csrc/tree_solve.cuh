@@ -11,22 +11,9 @@
 // record of the next round before waiting at the barrier.
 #pragma once
 
-#include "common.cuh"
+#include "units.cuh"
 
 namespace grass {
-
-template <typename T>
-struct PackT;
-template <>
-struct PackT<float> {
-    using V2 = float2;
-    using V4 = float4;
-};
-template <>
-struct PackT<double> {
-    using V2 = double2;
-    using V4 = Dbl4;
-};
 
 template <typename T>
 struct TreeKArgs {
@@ -46,6 +33,7 @@ struct TreeKArgs {
     unsigned int *bar;
     long long budget;
     int *err;
+    UnitArgs<T> u;        // the unit form (u.nl > 0), else the rounds above
 };
 
 template <typename T, int R>
@@ -320,7 +308,7 @@ __device__ __forceinline__ double run_bwd(const BwdBatch<T> &b, T *V, int64_t ba
 // solve (the solve's tail waits on __syncthreads after it).
 template <typename T, int R>
 __device__ inline void tree_tail_stage(const TreeKArgs<T> &a, T *ys) {
-    if (blockIdx.x != 0 || a.K1 >= a.rounds) return;
+    if (a.u.nl > 0 || blockIdx.x != 0 || a.K1 >= a.rounds) return;
     const TailSmem<T, R> sm(ys, a.ntl, a.tnf, a.tnb, a.ntc);
     for (int64_t i = threadIdx.x; i < a.tnf; i += blockDim.x) {
         sm.frec[i] = a.fwd_loc[a.tf0 - a.r0 + i];
@@ -340,10 +328,13 @@ __device__ inline void tree_tail_stage(const TreeKArgs<T> &a, T *ys) {
 // Solve in place on Y (n x R).  Called by every thread of a cooperative
 // grid; returns false when a barrier wait ran out (the caller must return).
 // mx accumulates max |x| over the values this thread wrote.  Ends without
-// a trailing grid barrier.
-template <typename T, int R, bool TRACK = true>
+// a trailing grid barrier.  B (unit form only): the right-hand side when it
+// is not in Y.  UNITS: the tree has the unit form (else the rounds).
+template <typename T, int R, bool TRACK, bool UNITS>
 __device__ __forceinline__ bool tree_solve_dev(const TreeKArgs<T> &a, T *Y, unsigned int &epoch,
-                                      double &mx, T *ys) {
+                                      double &mx, T *ys, const T *B = nullptr) {
+    if constexpr (UNITS)
+        return unit_solve_dev<T, R, TRACK>(a.u, a.bar, a.budget, a.err, B ? B : Y, Y, epoch, mx, ys);
     constexpr int TPR = Lay<R>::TPR;
     __shared__ int64_t s_roff[kMaxRounds + 1], s_eoff[kMaxRounds + 1];
     const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -992,6 +983,48 @@ inline int coop_grid(grass_ctx_t ctx, K kernel, int threads, size_t smem, int64_
 template <typename T, int R>
 inline TreeKArgs<T> tree_kargs(grass_ctx_t ctx, const grass_tree_s *Tr, const TreeFactor &f,
                                size_t *smem) {
+    TreeKArgs<T> ka;
+    std::memset((void *)&ka, 0, sizeof(ka));
+    ka.bar = ctx->gbar.p;
+    ka.budget = ctx->wait_budget;
+    ka.err = ctx->flags.p + 3;
+    const UnitTree &U = Tr->units;
+    if (U.built) {
+        ka.u.nl = (int)U.lv.size();
+        int local = 0, elim = 0;
+        for (int l = 0; l < ka.u.nl; ++l) {
+            const UnitLevel &L = U.lv[l];
+            auto &d = ka.u.lv[l];
+            d.n = L.n;
+            d.B = L.B;
+            d.nu = L.nu;
+            d.ord = l == 0 ? L.ord : nullptr;
+            d.meta = L.meta;
+            d.roff = L.roff;
+            d.cbeg = L.cbeg;
+            d.clist = L.cpos;
+            d.epos = L.epos;
+            d.edst = L.edst;
+            d.sptr = L.sptr;
+            d.V = reinterpret_cast<T *>(L.V);
+            d.exp = reinterpret_cast<T *>(L.exp);
+            if constexpr (sizeof(T) == 8) {
+                d.coef = f.unit.c64[l];
+                d.cm = f.unit.m64[l];
+            } else {
+                d.coef = f.unit.c32[l];
+                d.cm = f.unit.m32[l];
+            }
+            if (l + 1 < ka.u.nl) {
+                local = std::max(local, L.local);
+                elim = std::max(elim, L.elim);
+            }
+        }
+        if constexpr (sizeof(T) == 8) ka.u.rinv = f.unit.rinv64;
+        else ka.u.rinv = f.unit.rinv32;
+        *smem = unit_shape<T, R>(ka.u, local, elim, U.lv.back().local, U.lv.back().elim);
+        return ka;
+    }
     const TreeSchedule &S = Tr->sched;
     auto alive_at = [&](int k) { return S.tail_n - (S.elim_off[k] - S.elim_off[S.tail_k0]); };
     // the tail's rows and its records / coefficients must fit the budget,
@@ -1007,7 +1040,6 @@ inline TreeKArgs<T> tree_kargs(grass_ctx_t ctx, const grass_tree_s *Tr, const Tr
         ++K1;
     const int64_t ntl = alive_at(K1);
     *smem = tail_bytes(K1);
-    TreeKArgs<T> ka;
     ka.rounds = S.rounds;
     ka.K1 = K1;
     ka.base = S.tail_n - ntl;
@@ -1043,9 +1075,6 @@ inline TreeKArgs<T> tree_kargs(grass_ctx_t ctx, const grass_tree_s *Tr, const Tr
     if constexpr (sizeof(T) == 8) ka.root_invd = f.rinv64.p;
     else ka.root_invd = f.rinv32.p;
     ka.nroots = (int)Tr->nroots;
-    ka.bar = ctx->gbar.p;
-    ka.budget = ctx->wait_budget;
-    ka.err = ctx->flags.p + 3;
     return ka;
 }
 
