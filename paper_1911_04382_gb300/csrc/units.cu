@@ -255,25 +255,61 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_unit_build(UnitBuildArgs a
         }
         __syncthreads();
     }
-    // order by (round, position); the survivors last
-    int nel = 0, run = 0;
-    uint16_t *ro = a.roff + (int64_t)u * (kUnitRounds + 2);
-    for (int k = 0; k <= rounds; ++k) {
-        if (tid == 0) ro[k] = (uint16_t)run;
-        if (k == rounds) nel = run;
-        for (int i0 = 0; i0 < size; i0 += nt) {
-            const int i = i0 + tid;
-            const bool in = i < size && (k < rounds ? er[i] == k : er[i] == 255);
-            int tot;
-            const int at = run + un_scan(in ? 1 : 0, &tot);
-            if (in) {
-                pos[i] = (uint16_t)at;
-                own[at] = (uint16_t)i;
+    // Order by (round, one or two neighbours, list length, position), the
+    // survivors last: a warp's items of a round then run through the same
+    // branches and list lengths (an FP64 instruction occupies its pipe for
+    // the whole warp, however few lanes are on).  A bitonic sort of keys.
+    for (int j = tid; j < local; j += nt) cnt[j] = 0;
+    __syncthreads();
+    for (int i = tid; i < size; i += nt) {
+        if (er[i] == 255) continue;
+        atomicAdd(cnt + n1[i], 1);
+        if (n2[i] != 0xffff) atomicAdd(cnt + n2[i], 1);
+    }
+    __syncthreads();
+    int P = 1;
+    while (P < size) P <<= 1;
+    for (int i = tid; i < P; i += nt) {
+        uint32_t key = 0xffffffffu;
+        if (i < size) {
+            const uint32_t r = er[i];
+            key = r << 24 | (r == 255 ? 0u : (n2[i] != 0xffff ? 1u : 0u) << 23 |
+                                                 (uint32_t)min(cnt[i], 127) << 16) | (uint32_t)i;
+        }
+        beg[i] = (int32_t)key;
+    }
+    __syncthreads();
+    for (int k = 2; k <= P; k <<= 1)
+        for (int d = k >> 1; d > 0; d >>= 1) {
+            for (int i = tid; i < P; i += nt) {
+                const int x = i ^ d;
+                if (x <= i) continue;
+                const uint32_t a0 = (uint32_t)beg[i], a1 = (uint32_t)beg[x];
+                if ((a0 > a1) == ((i & k) == 0)) {
+                    beg[i] = (int32_t)a1;
+                    beg[x] = (int32_t)a0;
+                }
             }
-            run += tot;
+            __syncthreads();
+        }
+    int nel = size;
+    uint16_t *ro = a.roff + (int64_t)u * (kUnitRounds + 2);
+    __shared__ int s_nel;
+    if (tid == 0) s_nel = size;
+    __syncthreads();
+    for (int p = tid; p < size; p += nt) {
+        const uint32_t key = (uint32_t)beg[p];
+        const int i = (int)(key & 0xffffu), r = (int)(key >> 24);
+        pos[i] = (uint16_t)p;
+        own[p] = (uint16_t)i;
+        if (p == 0 || (int)((uint32_t)beg[p - 1] >> 24) != r) {
+            if (r == 255) s_nel = p;
+            else ro[r] = (uint16_t)p;
         }
     }
     __syncthreads();
+    nel = s_nel;
+    if (tid == 0) ro[rounds] = (uint16_t)nel;
     auto ref = [&](int x) { return x < size ? (int)pos[x] : x; };
     for (int p = tid; p < size; p += nt) {
         const int i = own[p];
@@ -572,7 +608,7 @@ bool unit_build(grass_ctx_t ctx, grass_tree_t T, UnitTree &U) {
            (const int32_t *)pos, (const int32_t *)E.par.p, (const int32_t *)E.ein.p,
            (const double *)E.pw.p, parent, U.w0);
     GCK(cudaFuncSetAttribute((const void *)k_unit_build, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kTailSmem));
+                             (int)unit_build_smem(kUnitTop)));
     GCK(cudaFuncSetAttribute((const void *)k_unit_factor, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kTailSmem));
     auto *up = tmp.get<int32_t>(n);

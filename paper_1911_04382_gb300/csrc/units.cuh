@@ -69,18 +69,21 @@ struct UnitArgs {
     UnitLevelArgs<T> lv[kUnitLevels];
 };
 
-// Columns per task.  FP32: 8 (32-byte row pieces, so that two units of 16
-// columns' rows fit an SM's shared memory side by side); FP64: 2.  The last
-// level, one block per column group: 4 or 1.
+// Columns worked on at a time (CG; the last level, one block per column
+// group: TG): rows of 64 bytes where they fit beside the lists.  Measured,
+// 1M vertices: 16 FP32 columns at once 131 us a solve, 8 at a time (two
+// units side by side) 143, 8 at a time with the next 8 loaded meanwhile 177;
+// 8 FP64 columns at once 217 us, 4 at a time 325.
 template <typename T, int R>
 struct UnitCols {
-    static constexpr int CG = sizeof(T) == 4 ? (R > 8 ? 8 : R) : (R > 2 ? 2 : R);
+    static constexpr int CG = sizeof(T) == 4 ? (R == 24 ? 8 : R > 16 ? 16 : R) : (R > 8 ? 8 : R);
+    static constexpr int NG = R / CG;
     static constexpr int TG = sizeof(T) == 4 ? (R > 4 ? 4 : R) : 1;
 };
 
-// Shared memory of one unit: the rows, then either the forward pass's
-// multipliers, contributors and list starts, or the backward pass's
-// coefficients.
+// Shared memory of one unit: the forward pass's multipliers, contributors
+// and list starts, or the backward pass's coefficients, in one region; then
+// the rows.
 template <typename T>
 struct UnitSmem {
     T *y;
@@ -89,23 +92,24 @@ struct UnitSmem {
     uint16_t *cl, *cb;
     __host__ __device__ static size_t up(size_t x) { return (x + 31) & ~size_t(31); }
     // the staged arrays are copied in whole 16-byte pieces: each is rounded up
-    __device__ UnitSmem(void *p, int local, int elim, int cg) {
-        char *q = reinterpret_cast<char *>(p);
-        y = reinterpret_cast<T *>(q);
-        size_t o = up((size_t)local * cg * sizeof(T));
-        cf = reinterpret_cast<typename PackT<T>::V4 *>(q + o);
-        cm = reinterpret_cast<T *>(q + o);
-        o = up(o + 2 * (size_t)elim * sizeof(T));
-        cl = reinterpret_cast<uint16_t *>(q + o);
-        o = up(o + 2 * (size_t)elim * sizeof(uint16_t));
-        cb = reinterpret_cast<uint16_t *>(q + o);
-    }
-    __host__ __device__ static size_t bytes(int local, int elim, int cg) {
-        const size_t y = up((size_t)local * cg * sizeof(T));
+    __host__ __device__ static size_t lists(int local, int elim) {
         const size_t f = up(2 * (size_t)elim * sizeof(T)) + up(2 * (size_t)elim * sizeof(uint16_t)) +
                          up(((size_t)local + 1) * sizeof(uint16_t));
         const size_t b = up((size_t)elim * sizeof(typename PackT<T>::V4));
-        return y + (f > b ? f : b);
+        return f > b ? f : b;
+    }
+    __host__ __device__ static size_t rows(int local, int cg) {
+        return up((size_t)local * cg * sizeof(T));
+    }
+    __device__ UnitSmem(void *p, int local, int elim) {
+        char *q = reinterpret_cast<char *>(p);
+        cf = reinterpret_cast<typename PackT<T>::V4 *>(q);
+        cm = reinterpret_cast<T *>(q);
+        size_t o = up(2 * (size_t)elim * sizeof(T));
+        cl = reinterpret_cast<uint16_t *>(q + o);
+        o = up(o + 2 * (size_t)elim * sizeof(uint16_t));
+        cb = reinterpret_cast<uint16_t *>(q + o);
+        y = reinterpret_cast<T *>(q + lists(local, elim));
     }
 };
 
@@ -114,8 +118,10 @@ struct UnitSmem {
 // last.
 template <typename T, int R>
 inline size_t unit_shape(UnitArgs<T> &a, int local, int elim, int tlocal, int telim) {
-    const size_t top = UnitSmem<T>::bytes(tlocal, telim, UnitCols<T, R>::TG);
-    const size_t one = a.nl > 1 ? UnitSmem<T>::bytes(local, elim, UnitCols<T, R>::CG) : 32;
+    using C = UnitCols<T, R>;
+    const size_t top = UnitSmem<T>::lists(tlocal, telim) + UnitSmem<T>::rows(tlocal, C::TG);
+    const size_t one = a.nl > 1 ? UnitSmem<T>::lists(local, elim) + UnitSmem<T>::rows(local, C::CG)
+                                : 32;
     a.groups = 4 * one <= kTailSmem ? 4 : 2 * one <= kTailSmem ? 2 : 1;
     a.gbytes = (int)one;
     const size_t all = one * a.groups;
@@ -188,7 +194,12 @@ __device__ __forceinline__ void cp_async(void *dst, const void *src) {
         asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(BYTES)
                      : "memory");
 }
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// all but the last N committed groups have arrived
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
 
 // bytes (rounded up to 16) from a 16-byte aligned array
 __device__ __forceinline__ void unit_copy(const UnitGroup &g, void *dst, const void *src, int bytes) {
@@ -255,6 +266,7 @@ __device__ __forceinline__ void unit_gather_sp(const UnitGroup &g, const UnitSme
         T acc[V];
 #pragma unroll
         for (int x = 0; x < V; ++x) acc[x] = (T)0;
+        if (mine && k == 0) uld<T, V>(s.y + p * CG + c, true, acc);
         if (mine) {
             // NB entries' loads before the first product
             constexpr int NB = SP == 1 ? 4 : 2;
@@ -282,13 +294,7 @@ __device__ __forceinline__ void unit_gather_sp(const UnitGroup &g, const UnitSme
 #pragma unroll
             for (int x = 0; x < V; ++x) acc[x] += __shfl_xor_sync(0xffffffffu, acc[x], d);
         }
-        if (mine && k == 0) {
-            T yv[V];
-            uld<T, V>(s.y + p * CG + c, true, yv);
-#pragma unroll
-            for (int x = 0; x < V; ++x) yv[x] += acc[x];
-            ust<T, V>(s.y + p * CG + c, true, yv);
-        }
+        if (mine && k == 0) ust<T, V>(s.y + p * CG + c, true, acc);
     }
 }
 
@@ -319,47 +325,45 @@ __device__ __forceinline__ void unit_gather(const UnitGroup &g, const UnitSmem<T
     g.sync();
 }
 
-// Stage a unit's lists and rows and load the own vertices' values: from the
-// vector (level 0), or the sums of the previous level's exports (a long list
-// by a warp).  Ends with the group's barrier.
-template <typename T, int R, int CG>
-__device__ __forceinline__ void unit_load(const UnitGroup &g, const UnitLevelArgs<T> &L, const T *E,
-                                          int u, const int4 m, const UnitSmem<T> &s,
-                                          uint16_t *s_roff, const T *Y, bool al, int c0) {
-    constexpr int V = UnitVec<T, CG>::V, LP = UnitVec<T, CG>::LP;
-    const int tid = g.tid, nt = g.nt, rounds = m.z & 0xffff;
-    const int size = (int)min((int64_t)L.B, L.n - (int64_t)u * L.B);
+// Stage a unit's lists and round offsets (asynchronous copies).
+template <typename T>
+__device__ __forceinline__ void unit_lists(const UnitGroup &g, const UnitLevelArgs<T> &L, int u,
+                                           const int4 m, const UnitSmem<T> &s, uint16_t *s_roff) {
+    const int64_t lo = (int64_t)u * unit_stride(L.B);
     const uint16_t *ro = L.roff + (int64_t)u * (kUnitRounds + 2);
-    const int64_t lo = (int64_t)u * unit_stride(L.B), pos0 = (int64_t)u * L.B;
     unit_copy(g, s.cb, L.cbeg + lo, (m.y + 1) * (int)sizeof(uint16_t));
-    if (Y) unit_rows<T, R, CG>(g, s, L.ord + pos0, 0, size, Y + c0, al);
     const int nc = L.cbeg[lo + m.y];
     unit_copy(g, s.cl, L.clist + lo, nc * (int)sizeof(uint16_t));
     unit_copy(g, s.cm, L.cm + lo, nc * (int)sizeof(T));
-    for (int k = tid; k <= rounds; k += nt) s_roff[k] = ro[k];
-    if (!Y) {
-        for (int it = tid; it < size * LP; it += nt) {
-            const int p = it / LP, c = (it % LP) * V;
-            const int b = L.sptr[pos0 + p], e = L.sptr[pos0 + p + 1];
-            T acc[V];
+    for (int k = g.tid; k <= (m.z & 0xffff); k += g.nt) s_roff[k] = ro[k];
+}
+
+// Levels above 0: the unit's rows as the sums of the previous level's
+// exports (a long list by a warp).  Ends with the group's barrier.
+template <typename T, int R, int CG>
+__device__ __forceinline__ void unit_sums(const UnitGroup &g, const UnitLevelArgs<T> &L, const T *E,
+                                          int u, const UnitSmem<T> &s, int c0) {
+    constexpr int V = UnitVec<T, CG>::V, LP = UnitVec<T, CG>::LP;
+    const int64_t pos0 = (int64_t)u * L.B;
+    const int size = (int)min((int64_t)L.B, L.n - pos0);
+    for (int it = g.tid; it < size * LP; it += g.nt) {
+        const int p = it / LP, c = (it % LP) * V;
+        const int b = L.sptr[pos0 + p], e = L.sptr[pos0 + p + 1];
+        T acc[V];
 #pragma unroll
-            for (int x = 0; x < V; ++x) acc[x] = (T)0;
-            if (e - b <= kUnitHeavy) {
-                for (int j = b; j < e; ++j) {
-                    T v[V];
-                    uld<T, V>(E + (int64_t)j * R + c0 + c, true, v);
+        for (int x = 0; x < V; ++x) acc[x] = (T)0;
+        if (e - b <= kUnitHeavy) {
+            for (int j = b; j < e; ++j) {
+                T v[V];
+                uld<T, V>(E + (int64_t)j * R + c0 + c, true, v);
 #pragma unroll
-                    for (int x = 0; x < V; ++x) acc[x] += v[x];
-                }
+                for (int x = 0; x < V; ++x) acc[x] += v[x];
             }
-            ust<T, V>(s.y + p * CG + c, true, acc);
         }
+        ust<T, V>(s.y + p * CG + c, true, acc);
     }
-    for (int it = tid; it < (m.y - size) * CG; it += nt) s.y[size * CG + it] = (T)0;
-    cp_async_wait();
     g.sync();
-    if (Y) return;
-    const int lane = tid & 31;
+    const int lane = g.tid & 31;
     unit_heavy(g, 0, size, [&](int p) { return L.sptr[pos0 + p + 1] - L.sptr[pos0 + p]; }, [&](int p) {
         const int b = L.sptr[pos0 + p], e = L.sptr[pos0 + p + 1];
         for (int c = 0; c < CG; ++c) {
@@ -429,13 +433,14 @@ __device__ __forceinline__ void unit_backward(const UnitGroup &g, const UnitSmem
             T y[V], a[V], b[V];
             uld<T, V>(s.y + p * CG + c, true, y);
             uld<T, V>(s.y + n1 * CG + c, true, a);
+#pragma unroll
+            for (int x = 0; x < V; ++x) b[x] = (T)0;
+            if (n2 != 0xffff) uld<T, V>(s.y + n2 * CG + c, true, b);
+#pragma unroll
+            for (int x = 0; x < V; ++x) y[x] = cf.x * y[x] + cf.y * a[x];
             if (n2 != 0xffff) {
-                uld<T, V>(s.y + n2 * CG + c, true, b);
 #pragma unroll
-                for (int x = 0; x < V; ++x) y[x] = cf.x * y[x] + cf.y * a[x] + cf.z * b[x];
-            } else {
-#pragma unroll
-                for (int x = 0; x < V; ++x) y[x] = cf.x * y[x] + cf.y * a[x];
+                for (int x = 0; x < V; ++x) y[x] += cf.z * b[x];
             }
             ust<T, V>(s.y + p * CG + c, true, y);
         }
@@ -448,15 +453,18 @@ __device__ __forceinline__ void unit_backward(const UnitGroup &g, const UnitSmem
 // this thread wrote.  Ends without a trailing grid barrier.
 // A block's thread groups take units side by side (the rounds of one unit
 // are a chain of short dependent steps: two to four chains at a time hide
-// each other's latency).  A group takes its units of a level in order forward
-// and in reverse backward, so the last one is still in shared memory when
-// the backward pass starts, unless the block solved a column group of the
-// last level in between (those go to the last blocks of the grid).
+// each other's latency).  A task is a unit with `span` of its column groups:
+// all of them when there are units enough for the grid (the lists are staged
+// once), one when there are not.  A group takes its tasks of a level in
+// order forward and in reverse backward, so the last column group it solved
+// is still in shared memory when the backward pass starts, unless the
+// block solved a column group of the last level in between (those go to the
+// last blocks of the grid).
 template <typename T, int R, bool TRACK>
 __device__ __forceinline__ bool unit_solve_dev(const UnitArgs<T> &a, unsigned int *bar,
                                                long long budget, int *err, const T *B, T *Y,
                                                unsigned int &epoch, double &mx, T *ys) {
-    constexpr int CG = UnitCols<T, R>::CG, NG = R / CG;
+    constexpr int CG = UnitCols<T, R>::CG, NG = UnitCols<T, R>::NG;
     constexpr int TG = UnitCols<T, R>::TG, NT = R / TG;
     constexpr int V = UnitVec<T, CG>::V, LP = UnitVec<T, CG>::LP;
     __shared__ uint16_t s_roff_all[4][kUnitRounds + 2];
@@ -470,11 +478,7 @@ __device__ __forceinline__ bool unit_solve_dev(const UnitArgs<T> &a, unsigned in
     const int gi = (int)threadIdx.x / g.nt;
     g.tid = (int)threadIdx.x - gi * g.nt;
     g.id = 1 + gi;
-    // Tasks (unit, column group) to groups: the column groups of a unit side
-    // by side in one block (its lists and the other halves of its rows are
-    // then in this SM's L1 or on their way), its other units G apart.
-    const int side = NG % groups == 0 ? groups : groups % NG == 0 ? NG : 1;
-    const int GG = G * groups, mg = me * side + gi % side + (gi / side) * (G * side);
+    const int GG = G * groups, mg = me + gi * G;
     uint16_t *s_roff = s_roff_all[gi];
     char *gsm = reinterpret_cast<char *>(ys) + (size_t)gi * a.gbytes;
     T tm = (T)0;
@@ -483,28 +487,43 @@ __device__ __forceinline__ bool unit_solve_dev(const UnitArgs<T> &a, unsigned in
     for (int l = 0; l < top; ++l) {
         const UnitLevelArgs<T> &L = a.lv[l];
         const T *E = l > 0 ? a.lv[l - 1].exp : nullptr;
-        for (int t = mg; t < L.nu * NG; t += GG) {
-            const int u = t / NG, c0 = (t % NG) * CG;
+        const int span = L.nu >= GG ? NG : 1, parts = NG / span;
+        for (int t = mg; t < L.nu * parts; t += GG) {
+            const int u = t / parts, cg0 = (t % parts) * span;
             const int4 m = L.meta[u];
-            const UnitSmem<T> s(gsm, m.y, m.x, CG);
-            unit_load<T, R, CG>(g, L, E, u, m, s, s_roff, l == 0 ? B : (const T *)nullptr, al, c0);
-            unit_forward<T, CG>(g, s, m, s_roff);
-            for (int it = g.tid; it < (m.y - m.x) * LP; it += g.nt) {
-                const int j = it / LP, c = (it % LP) * V;
-                T v[V];
-                uld<T, V>(s.y + (m.x + j) * CG + c, true, v);
-                ust<T, V>(L.exp + (int64_t)L.edst[m.w + j] * R + c0 + c, true, v);
-            }
-            if (top == 1 && t + GG >= L.nu * NG && me < G - NT) {
-                kept = true;   // stays in shared memory
-                continue;
-            }
+            const int size = (int)min((int64_t)L.B, L.n - (int64_t)u * L.B);
             const int32_t *ord = l == 0 ? L.ord + (int64_t)u * L.B : nullptr;
-            T *W = l == 0 ? Y : L.V + (int64_t)u * L.B * R;
-            // level 0's first round is as it was in B
-            const int p0 = l == 0 && (m.z & 0xffff) > 0 ? s_roff[1] : 0;
-            unit_store<T, R, CG>(g, s, ord, p0, m.x, W + c0, l == 0 ? al : true);
-            g.sync();
+            const UnitSmem<T> s(gsm, m.y, m.x);
+            unit_lists(g, L, u, m, s, s_roff);
+            if (l == 0) unit_rows<T, R, CG>(g, s, ord, 0, size, B + cg0 * CG, al);
+            cp_async_commit();
+            for (int k = 0; k < span; ++k) {
+                const int c0 = (cg0 + k) * CG;
+                if (l == 0 && k > 0) {
+                    unit_rows<T, R, CG>(g, s, ord, 0, size, B + c0, al);
+                    cp_async_commit();
+                }
+                cp_async_wait<0>();
+                for (int it = g.tid; it < (m.y - size) * CG; it += g.nt) s.y[size * CG + it] = (T)0;
+                if (l == 0) g.sync();
+                else unit_sums<T, R, CG>(g, L, E, u, s, c0);
+                unit_forward<T, CG>(g, s, m, s_roff);
+                for (int it = g.tid; it < (m.y - m.x) * LP; it += g.nt) {
+                    const int j = it / LP, c = (it % LP) * V;
+                    T v[V];
+                    uld<T, V>(s.y + (m.x + j) * CG + c, true, v);
+                    ust<T, V>(L.exp + (int64_t)L.edst[m.w + j] * R + c0 + c, true, v);
+                }
+                if (top == 1 && k + 1 == span && t + GG >= L.nu * parts && me < G - NT) {
+                    kept = true;   // stays in shared memory
+                    break;
+                }
+                T *W = l == 0 ? Y : L.V + (int64_t)u * L.B * R;
+                // level 0's first round is as it was in B
+                const int p0 = l == 0 && (m.z & 0xffff) > 0 ? s_roff[1] : 0;
+                unit_store<T, R, CG>(g, s, ord, p0, m.x, W + c0, l == 0 ? al : true);
+                g.sync();
+            }
         }
         if (!grid_sync(bar, budget, err, epoch)) return false;
     }
@@ -512,7 +531,6 @@ __device__ __forceinline__ bool unit_solve_dev(const UnitArgs<T> &a, unsigned in
     {
         constexpr int TV = UnitVec<T, TG>::V, TLP = UnitVec<T, TG>::LP;
         const UnitLevelArgs<T> &L = a.lv[top];
-        const T *E = top > 0 ? a.lv[top - 1].exp : nullptr;
         T *W = top > 0 ? L.V : Y;
         const bool wal = top > 0 ? true : al;
         UnitGroup h;
@@ -522,15 +540,21 @@ __device__ __forceinline__ bool unit_solve_dev(const UnitArgs<T> &a, unsigned in
         for (int t = G - 1 - me; t < NT; t += G) {
             const int c0 = t * TG;
             const int4 m = L.meta[0];
-            const UnitSmem<T> s(ys, m.y, m.x, TG);
-            unit_load<T, R, TG>(h, L, E, 0, m, s, s_roff_all[0], top == 0 ? B : (const T *)nullptr,
-                                al, c0);
+            const int rounds = m.z & 0xffff;
+            const UnitSmem<T> s(ys, m.y, m.x);
+            unit_lists(h, L, 0, m, s, s_roff_all[0]);
+            if (top == 0) unit_rows<T, R, TG>(h, s, L.ord, 0, m.y, B + c0, al);
+            cp_async_commit();
+            if (top > 0) unit_sums<T, R, TG>(h, L, a.lv[top - 1].exp, 0, s, c0);
+            cp_async_wait<0>();
+            h.sync();
             unit_forward<T, TG>(h, s, m, s_roff_all[0]);
             unit_coef(h, L, 0, m, s);
+            cp_async_commit();
             if (h.tid < TG) s.y[m.x * TG + h.tid] *= *a.rinv;
-            cp_async_wait();
+            cp_async_wait<0>();
             h.sync();
-            unit_backward<T, TG>(h, s, s_roff_all[0], m.z & 0xffff);
+            unit_backward<T, TG>(h, s, s_roff_all[0], rounds);
             for (int it = h.tid; it < m.y * TLP; it += h.nt) {
                 const int p = it / TLP, c = (it % TLP) * TV;
                 T v[TV];
@@ -548,46 +572,58 @@ __device__ __forceinline__ bool unit_solve_dev(const UnitArgs<T> &a, unsigned in
         const UnitLevelArgs<T> &L = a.lv[l];
         const T *X = a.lv[l + 1].V;   // the next level's solution
         const bool wal = l == 0 ? al : true;
-        const int nt_l = L.nu * NG;
-        const int last = mg < nt_l ? mg + (nt_l - 1 - mg) / GG * GG : -1;
+        const int span = L.nu >= GG ? NG : 1, parts = NG / span;
+        const int ntask = L.nu * parts;
+        const int last = mg < ntask ? mg + (ntask - 1 - mg) / GG * GG : -1;
         if (kept) {   // the coefficients do not wait for the last level
-            const int u = last / NG;
+            const int u = last / parts;
             const int4 m = L.meta[u];
-            const UnitSmem<T> s(gsm, m.y, m.x, CG);
+            const UnitSmem<T> s(gsm, m.y, m.x);
             g.sync();
             unit_coef(g, L, u, m, s);
+            cp_async_commit();
         }
         if (!grid_sync(bar, budget, err, epoch)) return false;
         for (int t = last; t >= 0; t -= GG) {
-            const int u = t / NG, c0 = (t % NG) * CG;
+            const int u = t / parts, cg0 = (t % parts) * span;
             const int4 m = L.meta[u];
             const int rounds = m.z & 0xffff;
-            const UnitSmem<T> s(gsm, m.y, m.x, CG);
+            const int size = (int)min((int64_t)L.B, L.n - (int64_t)u * L.B);
             const int32_t *ord = l == 0 ? L.ord + (int64_t)u * L.B : nullptr;
             T *W = l == 0 ? Y : L.V + (int64_t)u * L.B * R;
-            const int size = (int)min((int64_t)L.B, L.n - (int64_t)u * L.B);
-            if (!(kept && t == last)) {
+            const UnitSmem<T> s(gsm, m.y, m.x);
+            const bool keep = kept && t == last;
+            int p1 = 0;
+            if (!keep) {
                 const uint16_t *ro = L.roff + (int64_t)u * (kUnitRounds + 2);
                 for (int k = g.tid; k <= rounds; k += g.nt) s_roff[k] = ro[k];
                 unit_coef(g, L, u, m, s);
-                const int p1 = l == 0 && rounds > 0 ? ro[1] : 0;
-                unit_rows<T, R, CG>(g, s, ord, 0, p1, B + c0, wal);
-                unit_rows<T, R, CG>(g, s, ord, p1, m.x, W + c0, wal);
+                p1 = l == 0 && rounds > 0 ? ro[1] : 0;
+            } else {
+                p1 = rounds > 0 ? s_roff[1] : 0;
             }
-            for (int it = g.tid; it < (m.y - m.x) * LP; it += g.nt) {
-                const int j = it / LP, c = (it % LP) * V;
-                T v[V];
-                uld<T, V>(X + (int64_t)L.epos[m.w + j] * R + c0 + c, true, v);
-                ust<T, V>(s.y + (m.x + j) * CG + c, true, v);
+            for (int k = span - 1; k >= 0; --k) {
+                const int c0 = (cg0 + k) * CG;
+                if (!keep || k + 1 < span) {
+                    unit_rows<T, R, CG>(g, s, ord, 0, p1, B + c0, wal);
+                    unit_rows<T, R, CG>(g, s, ord, p1, m.x, W + c0, wal);
+                    cp_async_commit();
+                }
+                for (int it = g.tid; it < (m.y - m.x) * LP; it += g.nt) {
+                    const int j = it / LP, c = (it % LP) * V;
+                    T v[V];
+                    uld<T, V>(X + (int64_t)L.epos[m.w + j] * R + c0 + c, true, v);
+                    ust<T, V>(s.y + (m.x + j) * CG + c, true, v);
+                }
+                cp_async_wait<0>();
+                g.sync();
+                unit_backward<T, CG>(g, s, s_roff, rounds);
+                unit_store<T, R, CG>(g, s, ord, 0, size, W + c0, wal);
+                if (TRACK) {
+                    for (int it = g.tid; it < size * CG; it += g.nt) tm = fmax(tm, fabs(s.y[it]));
+                }
+                g.sync();
             }
-            cp_async_wait();
-            g.sync();
-            unit_backward<T, CG>(g, s, s_roff, rounds);
-            unit_store<T, R, CG>(g, s, ord, 0, size, W + c0, wal);
-            if (TRACK) {
-                for (int it = g.tid; it < size * CG; it += g.nt) tm = fmax(tm, fabs(s.y[it]));
-            }
-            g.sync();
         }
     }
     if (TRACK) mx = fmax(mx, (double)tm);
