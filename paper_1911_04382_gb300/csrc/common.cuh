@@ -167,6 +167,7 @@ struct grass_ctx_s {
     int amg_sweeps = 1;         // Jacobi sweeps before and after each coarse correction
     int lmax_amg = 0;           // 1: lambda_max estimates solve L_S by multigrid-preconditioned CG
     grass::Arena amg_tmp;       // the multigrid setup's temporary arrays
+    grass::Arena core_tmp;      // the core form's
     int amg_fused = 1;          // 1: the multigrid PCG runs as one cooperative kernel (amg_fused.cu)
     int64_t amg_tail_n = 0;     // its levels of at most this many vertices run in one block
     int64_t amg_warp_n = 16384; // its levels of at most this many vertices take a warp per row
@@ -363,7 +364,7 @@ struct alignas(32) Dbl4 {
 // Unit form of a single tree's solve (units.cuh, units.cu): one level per
 // grid phase, the units of a level eliminated block by block.
 constexpr int kUnitMin = 256;       // smallest unit of a level with several units
-constexpr int kUnitMax = 2048;      // largest: 16 FP32 columns of it fit shared memory
+constexpr int kUnitMax = 1792;      // largest: 8 FP64 columns of it fit shared memory
 constexpr int kUnitTop = 3584;      // largest last level (one unit, few columns a block)
 constexpr int kUnitRounds = 62;     // block-local elimination rounds (about 14 needed)
 constexpr int kUnitLevels = 5;
@@ -386,8 +387,12 @@ struct UnitLevel {
 };
 struct UnitTree {
     bool built = false;
+    bool open = false;              // one level only; its survivors are left to the caller
     Arena arena;
-    double *w0 = nullptr;           // [n] level 0's weights to the parent, by position
+    // [n] preorder (heavy child last): position of a vertex, vertex and
+    // parent position of a position, weight to the parent
+    int32_t *pos = nullptr, *vid = nullptr, *parent = nullptr;
+    double *w0 = nullptr;
     std::vector<UnitLevel> lv;
 };
 struct UnitFactor {
@@ -398,6 +403,20 @@ struct UnitFactor {
     std::vector<float *> m32;
     double *rinv64 = nullptr;
     float *rinv32 = nullptr;
+};
+
+// The sparsifier's core (core.cu): S's matrix with everything eliminated that
+// the vertices of its added edges leave hanging or in a chain.
+struct CoreForm {
+    bool built = false;             // tried for the present S; usable when low.built
+    Arena arena;
+    UnitTree low, tree;             // the elimination (one open level), the core's own tree
+    UnitFactor low_f, tree_f;
+    int64_t n = 0, nnz = 0;
+    int32_t *vert = nullptr;        // [n] vertex of a core index
+    int32_t *ptr = nullptr, *col = nullptr;   // core adjacency (tree and added edges)
+    double *w64 = nullptr;
+    float *w32 = nullptr;
 };
 
 // Elimination schedule of the spanning tree by rake (degree 1) and compress
@@ -544,6 +563,7 @@ struct grass_sparsifier_s {
     grass::DBuf<int32_t> p_ptr, p_col;
     grass::DBuf<double> p_w64;
     grass::DBuf<float> p_w32;
+    std::unique_ptr<grass::CoreForm> core;        // built on first use after each change of S
     // multigrid hierarchies of L_S ([0]) and L_S + D ([1]), built on first
     // use after each change of S
     std::unique_ptr<grass::AmgHier> amg[2];
@@ -608,9 +628,28 @@ double tree_solve_bytes(const grass_tree_s *T, int r, double s);
 
 // Builds U for T's tree; false when the tree keeps the elimination rounds.
 bool unit_build(grass_ctx_t ctx, grass_tree_t T, UnitTree &U);
-// Coefficients of L_T (D null) or L_T + D.
-void unit_factor(grass_ctx_t ctx, grass_tree_t T, const UnitTree &U, const double *D,
-                 UnitFactor &f);
+// The levels of a tree given by parents (preorder positions): every level,
+// or (pin: [n] vertices that must survive) the first one alone; false when the
+// tree is not suited.  core, parent: [n] on return the next level's index of
+// every survivor and, by that index, its parent; scnt: exports per index.
+bool unit_levels(grass_ctx_t ctx, int64_t n, int32_t *parent, const int32_t *vid, const uint8_t *pin,
+                 Arena &tmp, UnitTree &U, int32_t *core, int32_t **scnt, int64_t *n1);
+// The exports of level P grouped by the next level's order lidx ([n1], null:
+// by index).
+void unit_group(grass_ctx_t ctx, UnitTree &U, UnitLevel &P, int64_t n1, const int32_t *lidx,
+                const int32_t *scnt, Arena &tmp, int32_t *sptr);
+// Coefficients of the tree's matrix (D null) or with the load D; next_w: the
+// survivors' weights to their parents (U.open).
+void unit_factor(grass_ctx_t ctx, const UnitTree &U, const double *D, UnitFactor &f,
+                 double *next_w = nullptr);
+
+// ---------------------------------------------------------------- core.cu
+
+// X = L_S^{-1} Y (grounded) by CG on the core; false when S has no core form
+// (the caller takes the CG over all vertices).  Arguments as s_solve.
+bool core_solve(grass_ctx_t ctx, grass_sparsifier_t S, int r, grass_prec prec, const void *Y, void *X,
+                double tol, int maxit, unsigned long long *maxbits);
+
 // In-place tree solve of the n x r block Y (prec), or from B into Y;
 // optionally tracks the max |x| bit pattern into maxbits (device, uint64 for
 // both precisions).

@@ -98,6 +98,7 @@ void sparsifier_rebuild(grass_ctx_t ctx, grass_sparsifier_t S) {
         S->s_heavy.count = 0;
     }
     S->pre_ok = false;
+    S->core.reset();
     S->amg[0].reset();
     S->amg[1].reset();
 }

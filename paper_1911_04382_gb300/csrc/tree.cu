@@ -488,7 +488,7 @@ void tree_factor(grass_ctx_t ctx, grass_tree_t T, bool with_D, TreeFactor &f) {
     const TreeSchedule &S = T->sched;
     const int64_t n = g.n;
     if (T->units.built) {
-        unit_factor(ctx, T, T->units, with_D ? g.D64.p : nullptr, f.unit);
+        unit_factor(ctx, T->units, with_D ? g.D64.p : nullptr, f.unit);
         return;
     }
     f.invd64.alloc(n);

@@ -978,6 +978,49 @@ inline int coop_grid(grass_ctx_t ctx, K kernel, int threads, size_t smem, int64_
     return (int)std::min<int64_t>(full, need);
 }
 
+// Kernel arguments of the unit form U with factor f, and the dynamic shared
+// memory R columns need.
+template <typename T, int R>
+inline UnitArgs<T> unit_args(const UnitTree &U, const UnitFactor &f, size_t *smem) {
+    UnitArgs<T> a;
+    std::memset((void *)&a, 0, sizeof(a));
+    a.nl = (int)U.lv.size();
+    int local = 0, elim = 0;
+    for (int l = 0; l < a.nl; ++l) {
+        const UnitLevel &L = U.lv[l];
+        auto &d = a.lv[l];
+        d.n = L.n;
+        d.B = L.B;
+        d.nu = L.nu;
+        d.ord = l == 0 ? L.ord : nullptr;
+        d.meta = L.meta;
+        d.roff = L.roff;
+        d.cbeg = L.cbeg;
+        d.clist = L.cpos;
+        d.epos = L.epos;
+        d.edst = L.edst;
+        d.sptr = L.sptr;
+        d.V = reinterpret_cast<T *>(L.V);
+        d.exp = reinterpret_cast<T *>(L.exp);
+        if constexpr (sizeof(T) == 8) {
+            d.coef = f.c64[l];
+            d.cm = f.m64[l];
+        } else {
+            d.coef = f.c32[l];
+            d.cm = f.m32[l];
+        }
+        if (l + 1 < a.nl || U.open) {
+            local = std::max(local, L.local);
+            elim = std::max(elim, L.elim);
+        }
+    }
+    if constexpr (sizeof(T) == 8) a.rinv = f.rinv64;
+    else a.rinv = f.rinv32;
+    const UnitLevel &top = U.lv.back();
+    *smem = unit_shape<T, R>(a, local, elim, U.open ? 0 : top.local, U.open ? 0 : top.elim);
+    return a;
+}
+
 // Host side: the arguments of one solve on tree T with factor f, and the
 // dynamic shared memory its tail needs.
 template <typename T, int R>
@@ -988,41 +1031,8 @@ inline TreeKArgs<T> tree_kargs(grass_ctx_t ctx, const grass_tree_s *Tr, const Tr
     ka.bar = ctx->gbar.p;
     ka.budget = ctx->wait_budget;
     ka.err = ctx->flags.p + 3;
-    const UnitTree &U = Tr->units;
-    if (U.built) {
-        ka.u.nl = (int)U.lv.size();
-        int local = 0, elim = 0;
-        for (int l = 0; l < ka.u.nl; ++l) {
-            const UnitLevel &L = U.lv[l];
-            auto &d = ka.u.lv[l];
-            d.n = L.n;
-            d.B = L.B;
-            d.nu = L.nu;
-            d.ord = l == 0 ? L.ord : nullptr;
-            d.meta = L.meta;
-            d.roff = L.roff;
-            d.cbeg = L.cbeg;
-            d.clist = L.cpos;
-            d.epos = L.epos;
-            d.edst = L.edst;
-            d.sptr = L.sptr;
-            d.V = reinterpret_cast<T *>(L.V);
-            d.exp = reinterpret_cast<T *>(L.exp);
-            if constexpr (sizeof(T) == 8) {
-                d.coef = f.unit.c64[l];
-                d.cm = f.unit.m64[l];
-            } else {
-                d.coef = f.unit.c32[l];
-                d.cm = f.unit.m32[l];
-            }
-            if (l + 1 < ka.u.nl) {
-                local = std::max(local, L.local);
-                elim = std::max(elim, L.elim);
-            }
-        }
-        if constexpr (sizeof(T) == 8) ka.u.rinv = f.unit.rinv64;
-        else ka.u.rinv = f.unit.rinv32;
-        *smem = unit_shape<T, R>(ka.u, local, elim, U.lv.back().local, U.lv.back().elim);
+    if (Tr->units.built) {
+        ka.u = unit_args<T, R>(Tr->units, f.unit, smem);
         return ka;
     }
     const TreeSchedule &S = Tr->sched;

@@ -440,11 +440,12 @@ __global__ void k_un_sptr(int n1, const int32_t *lidx, const int32_t *scnt, int3
     int run = 0;
     for (int p0 = 0; p0 < n1; p0 += blockDim.x) {
         const int p = p0 + threadIdx.x;
+        const int i = p < n1 && lidx ? lidx[p] : p;
         int t;
-        const int s = run + un_scan(p < n1 ? scnt[lidx[p]] : 0, &t);
+        const int s = run + un_scan(p < n1 ? scnt[i] : 0, &t);
         if (p < n1) {
             sptr[p] = cur[p] = s;
-            pos_of[lidx[p]] = p;
+            pos_of[i] = p;
         }
         run += t;
     }
@@ -578,51 +579,41 @@ int unit_size(int64_t n, int sms) {
 
 }  // namespace
 
-bool unit_build(grass_ctx_t ctx, grass_tree_t T, UnitTree &U) {
-    const EulerTour &E = T->euler;
-    const int64_t n = T->g.n;
-    U.lv.clear();
-    U.built = false;
-    if (!E.built || T->batch || T->nroots != 1 || ctx->num_sms <= 0 || n < 2) return false;
-    U.arena.chunk_min = (size_t)n * 40 + ((size_t)1 << 20);
-    Arena tmp;
-    tmp.chunk_min = (size_t)n * 72 + ((size_t)1 << 20);
-    // preorder with the heavy child last
-    auto *heavy = tmp.get<unsigned long long>(n);
-    auto *shift = tmp.get<int64_t>(E.L + 1);
-    auto *sum = tmp.get<int64_t>(E.L + 1);
-    auto *pos = tmp.get<int32_t>(n);
-    auto *vid = tmp.get<int32_t>(n);
-    auto *parent = tmp.get<int32_t>(n);
-    U.w0 = U.arena.get<double>(n);
-    memset_d(ctx, heavy, 0, n * sizeof(unsigned long long));
-    launch(ctx, k_un_heavy, cdiv(n, kBlock), kBlock, 0, n, (const int32_t *)E.ein.p,
-           (const int32_t *)E.eout.p, (const int32_t *)E.par.p, heavy);
-    launch(ctx, k_un_shift, cdiv(n, kBlock), kBlock, 0, n, T->ground, (const int32_t *)E.ein.p,
-           (const int32_t *)E.eout.p, (const int32_t *)E.par.p, (const int32_t *)E.pre.p,
-           (const unsigned long long *)heavy, shift);
-    scan_i64(ctx, shift, sum, E.L, nullptr);
-    launch(ctx, k_un_pos, cdiv(n, kBlock), kBlock, 0, n, (const int32_t *)E.ein.p,
-           (const int32_t *)E.pre.p, (const int64_t *)shift, (const int64_t *)sum, pos, vid);
-    launch(ctx, k_un_level0, cdiv(n, kBlock), kBlock, 0, n, (const int32_t *)vid,
-           (const int32_t *)pos, (const int32_t *)E.par.p, (const int32_t *)E.ein.p,
-           (const double *)E.pw.p, parent, U.w0);
+void unit_group(grass_ctx_t ctx, UnitTree &U, UnitLevel &P, int64_t n1, const int32_t *lidx,
+                const int32_t *scnt, Arena &tmp, int32_t *sptr) {
+    P.epos = U.arena.get<int32_t>(P.nexp);
+    P.edst = U.arena.get<int32_t>(P.nexp);
+    auto *cur = tmp.get<int32_t>(n1);
+    auto *pos_of = tmp.get<int32_t>(n1);
+    auto *raw = tmp.get<int32_t>(P.nexp);
+    launch(ctx, k_un_sptr, 1, 1024, 0, (int)n1, lidx, scnt, sptr, cur, pos_of);
+    launch(ctx, k_un_sfill, cdiv(P.nexp, kBlock), kBlock, 0, P.nexp, (const int32_t *)P.ecore,
+           (const int32_t *)pos_of, cur, raw, P.epos);
+    launch(ctx, k_un_ssort, cdiv(P.nexp, kBlock), kBlock, 0, P.nexp, (const int32_t *)P.epos,
+           (const int32_t *)sptr, (const int32_t *)raw, P.edst);
+}
+
+bool unit_levels(grass_ctx_t ctx, int64_t n, int32_t *parent, const int32_t *vid,
+                 const uint8_t *pin_in, Arena &tmp, UnitTree &U, int32_t *core, int32_t **scnt_out,
+                 int64_t *n_next) {
     GCK(cudaFuncSetAttribute((const void *)k_unit_build, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)unit_build_smem(kUnitTop)));
     GCK(cudaFuncSetAttribute((const void *)k_unit_factor, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kTailSmem));
     auto *up = tmp.get<int32_t>(n);
-    auto *core = tmp.get<int32_t>(n);
     auto *halo = tmp.get<int32_t>(n + kUnitTop);
     auto *pin = tmp.get<uint8_t>(n);
     auto *tot = tmp.get<int>(8);
     int64_t nl = n;
     int32_t *scnt = nullptr;
+    U.lv.clear();
+    U.built = false;
+    U.open = pin_in != nullptr;
     for (int l = 0; l < kUnitLevels; ++l) {
         U.lv.emplace_back();
         UnitLevel &L = U.lv.back();
         L.n = nl;
-        L.B = nl <= kUnitTop ? (int)nl : unit_size(nl, ctx->num_sms);
+        L.B = nl <= kUnitTop && !U.open ? (int)nl : unit_size(nl, ctx->num_sms);
         L.nu = (int)cdiv(nl, L.B);
         const int B = L.B, nu = L.nu;
         L.ord = U.arena.get<int32_t>(nl);
@@ -635,7 +626,8 @@ bool unit_build(grass_ctx_t ctx, grass_tree_t T, UnitTree &U) {
         L.cpos = U.arena.get<uint16_t>((size_t)nu * unit_stride(B));
         auto *cnt = tmp.get<int32_t>(2 * (size_t)nu);
         auto *soff = tmp.get<int32_t>(nu);
-        memset_d(ctx, pin, 0, nl);
+        if (pin_in) copy_d(ctx, pin, pin_in, nl);
+        else memset_d(ctx, pin, 0, nl);
         memset_d(ctx, tot, 0, 8 * sizeof(int));
         launch(ctx, k_un_cross, cdiv(nl, kBlock), kBlock, 0, nl, B, (const int32_t *)parent, pin);
         UnitBuildArgs a{nl, B, parent, pin, l == 0 ? vid : nullptr, L.ord, L.lidx, L.nn, L.meta,
@@ -643,20 +635,8 @@ bool unit_build(grass_ctx_t ctx, grass_tree_t T, UnitTree &U) {
         launch(ctx, k_unit_build, nu, kBuildThreads, unit_build_smem(B), a);
         launch(ctx, k_un_offsets, 1, 1024, 0, nu, (const int32_t *)cnt, soff, L.meta, tot);
         if (l > 0) {
-            // the previous level's exports, grouped by this level's positions
-            UnitLevel &P = U.lv[l - 1];
             L.sptr = U.arena.get<int32_t>(nl + 1);
-            P.epos = U.arena.get<int32_t>(P.nexp);
-            P.edst = U.arena.get<int32_t>(P.nexp);
-            auto *cur = tmp.get<int32_t>(nl);
-            auto *pos_of = tmp.get<int32_t>(nl);
-            auto *raw = tmp.get<int32_t>(P.nexp);
-            launch(ctx, k_un_sptr, 1, 1024, 0, (int)nl, (const int32_t *)L.lidx,
-                   (const int32_t *)scnt, L.sptr, cur, pos_of);
-            launch(ctx, k_un_sfill, cdiv(P.nexp, kBlock), kBlock, 0, P.nexp,
-                   (const int32_t *)P.ecore, (const int32_t *)pos_of, cur, raw, P.epos);
-            launch(ctx, k_un_ssort, cdiv(P.nexp, kBlock), kBlock, 0, P.nexp,
-                   (const int32_t *)P.epos, (const int32_t *)L.sptr, (const int32_t *)raw, P.edst);
+            unit_group(ctx, U, U.lv[l - 1], nl, L.lidx, scnt, tmp, L.sptr);
         }
         int h[4];
         d2h(ctx, h, tot, sizeof(h));
@@ -664,12 +644,15 @@ bool unit_build(grass_ctx_t ctx, grass_tree_t T, UnitTree &U) {
         L.nexp = h[1];
         L.local = h[2];
         L.elim = h[3];
-        if (nu == 1) {
+        if (nu == 1 && !U.open) {
             if (n1 != 1) return false;   // the round limit: keep the elimination rounds
             U.built = true;
             break;
         }
-        if (n1 > nl / 2 || L.local > kUnitMax + 128) return false;
+        // the widest column groups of a unit must fit shared memory
+        if (n1 > nl / 2 ||
+            UnitSmem<double>::lists(L.local, L.elim) + UnitSmem<double>::rows(L.local, 8) > kTailSmem)
+            return false;
         L.exp = U.arena.get<char>((size_t)L.nexp * 32 * sizeof(double));
         L.dexp = U.arena.get<double>(L.nexp);
         L.ecore = U.arena.get<int32_t>(L.nexp);
@@ -681,6 +664,10 @@ bool unit_build(grass_ctx_t ctx, grass_tree_t T, UnitTree &U) {
                (const int32_t *)halo, (const int32_t *)up, (const int32_t *)core, L.ecore, parent,
                scnt);
         nl = n1;
+        if (U.open) {
+            U.built = true;
+            break;
+        }
     }
     if (!U.built) return false;
     for (size_t l = 1; l < U.lv.size(); ++l) {
@@ -688,13 +675,53 @@ bool unit_build(grass_ctx_t ctx, grass_tree_t T, UnitTree &U) {
         L.V = U.arena.get<char>((size_t)L.n * 32 * sizeof(double));
         L.w = U.arena.get<double>(L.n);
     }
+    *scnt_out = scnt;
+    *n_next = nl;
+    return true;
+}
+
+bool unit_build(grass_ctx_t ctx, grass_tree_t T, UnitTree &U) {
+    const EulerTour &E = T->euler;
+    const int64_t n = T->g.n;
+    U.built = false;
+    if (!E.built || T->batch || T->nroots != 1 || ctx->num_sms <= 0 || n < 2) return false;
+    U.arena.chunk_min = (size_t)n * 52 + ((size_t)1 << 20);
+    Arena tmp;
+    tmp.chunk_min = (size_t)n * 64 + ((size_t)1 << 20);
+    // preorder with the heavy child last
+    auto *heavy = tmp.get<unsigned long long>(n);
+    auto *shift = tmp.get<int64_t>(E.L + 1);
+    auto *sum = tmp.get<int64_t>(E.L + 1);
+    auto *parent = tmp.get<int32_t>(n);
+    auto *core = tmp.get<int32_t>(n);
+    U.pos = U.arena.get<int32_t>(n);
+    U.vid = U.arena.get<int32_t>(n);
+    U.parent = U.arena.get<int32_t>(n);
+    U.w0 = U.arena.get<double>(n);
+    memset_d(ctx, heavy, 0, n * sizeof(unsigned long long));
+    launch(ctx, k_un_heavy, cdiv(n, kBlock), kBlock, 0, n, (const int32_t *)E.ein.p,
+           (const int32_t *)E.eout.p, (const int32_t *)E.par.p, heavy);
+    launch(ctx, k_un_shift, cdiv(n, kBlock), kBlock, 0, n, T->ground, (const int32_t *)E.ein.p,
+           (const int32_t *)E.eout.p, (const int32_t *)E.par.p, (const int32_t *)E.pre.p,
+           (const unsigned long long *)heavy, shift);
+    scan_i64(ctx, shift, sum, E.L, nullptr);
+    launch(ctx, k_un_pos, cdiv(n, kBlock), kBlock, 0, n, (const int32_t *)E.ein.p,
+           (const int32_t *)E.pre.p, (const int64_t *)shift, (const int64_t *)sum, U.pos, U.vid);
+    launch(ctx, k_un_level0, cdiv(n, kBlock), kBlock, 0, n, (const int32_t *)U.vid,
+           (const int32_t *)U.pos, (const int32_t *)E.par.p, (const int32_t *)E.ein.p,
+           (const double *)E.pw.p, U.parent, U.w0);
+    copy_d(ctx, parent, U.parent, n * sizeof(int32_t));
+    int32_t *scnt = nullptr;
+    int64_t n1 = 0;
+    if (!unit_levels(ctx, n, parent, U.vid, nullptr, tmp, U, core, &scnt, &n1)) return false;
     ctx->sync();   // the temporaries go
     return true;
 }
 
-void unit_factor(grass_ctx_t ctx, grass_tree_t T, const UnitTree &U, const double *D,
-                 UnitFactor &f) {
-    f.arena.chunk_min = (size_t)T->g.n * 76 + ((size_t)1 << 16);
+void unit_factor(grass_ctx_t ctx, const UnitTree &U, const double *D, UnitFactor &f,
+                 double *next_w) {
+    f.arena.chunk_min = (size_t)U.lv[0].n * 76 + ((size_t)1 << 16);
+    f.arena.reset();
     f.c64.clear();
     f.c32.clear();
     f.m64.clear();
@@ -707,11 +734,11 @@ void unit_factor(grass_ctx_t ctx, grass_tree_t T, const UnitTree &U, const doubl
         f.c32.push_back(f.arena.get<float4>(L.n));
         f.m64.push_back(f.arena.get<double>((size_t)L.nu * unit_stride(L.B)));
         f.m32.push_back(f.arena.get<float>((size_t)L.nu * unit_stride(L.B)));
-        const bool last = l + 1 == U.lv.size();
+        const bool end = l + 1 == U.lv.size(), last = end && !U.open;
         UnitFactorArgs a{L.n, L.B, L.meta, L.roff, L.cbeg, L.clist, L.cpos, f.m64[l], f.m32[l], L.nn, L.lidx, L.ord,
                          l == 0 ? U.w0 : L.w, l == 0 ? D : nullptr,
                          l > 0 && D ? U.lv[l - 1].dexp : nullptr, L.sptr, L.ecore, L.edst,
-                         last ? nullptr : U.lv[l + 1].w, L.dexp, f.c64[l], f.c32[l], f.rinv64,
+                         end ? next_w : U.lv[l + 1].w, L.dexp, f.c64[l], f.c32[l], f.rinv64,
                          f.rinv32, last ? 1 : 0};
         launch(ctx, k_unit_factor, L.nu, kBuildThreads, unit_factor_smem(L.local, L.elim), a);
     }

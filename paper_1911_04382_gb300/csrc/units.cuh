@@ -120,7 +120,7 @@ template <typename T, int R>
 inline size_t unit_shape(UnitArgs<T> &a, int local, int elim, int tlocal, int telim) {
     using C = UnitCols<T, R>;
     const size_t top = UnitSmem<T>::lists(tlocal, telim) + UnitSmem<T>::rows(tlocal, C::TG);
-    const size_t one = a.nl > 1 ? UnitSmem<T>::lists(local, elim) + UnitSmem<T>::rows(local, C::CG)
+    const size_t one = elim > 0 ? UnitSmem<T>::lists(local, elim) + UnitSmem<T>::rows(local, C::CG)
                                 : 32;
     a.groups = 4 * one <= kTailSmem ? 4 : 2 * one <= kTailSmem ? 2 : 1;
     a.gbytes = (int)one;

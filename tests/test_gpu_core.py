@@ -1,0 +1,89 @@
+"""CG on the sparsifier's core (csrc/core.cu) against the oracle's CG over
+all vertices: the same iterates, so the same embedding both when the solves
+converge and when every one ends at its iteration cap, on trees whose core is
+a single unit and several, with hubs, doubled edges' ends and every column
+count; and the sides of the rule that chooses it.
+
+Tolerances: FP64 1e-10 of the largest heat, as the other embedding tests (the
+capped iterates are those of exact arithmetic up to rounding on both sides);
+FP32 1e-3 as there.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from synth import graphs, rng
+from tests.gpu_util import dev, gpu_graph, host
+
+pytestmark = pytest.mark.gpu
+
+
+def _graph(kind):
+    if kind == "grid3d":
+        return graphs.grid3d_loguniform(22, 21, 20, seed=3)
+    if kind == "power":
+        return graphs.power_grid(70, seed=4)
+    if kind == "mesh":
+        return graphs.grid2d_uniform(181, 160, seed=5, lo=0.1, hi=10.0)
+    return graphs.chung_lu(6000, seed=6)
+
+
+@pytest.mark.parametrize("kind,every", [("grid3d", 97), ("power", 61), ("mesh", 211), ("mesh", 4001),
+                                        ("powerlaw", 401)])
+@pytest.mark.parametrize("maxit,tol", [(3000, 1e-13), (4, 1e-13)])
+@pytest.mark.parametrize("r", [2, 8, 16, 24])
+def test_core_embedding_matches_oracle(gpu, kind, every, maxit, tol, r):
+    import torch
+    g = _graph(kind)
+    og = oracle.from_graph(g)
+    rho = g.n // 2
+    ot = oracle.build_tree(og, rho)
+    off = np.flatnonzero(ot.in_tree == 0)
+    add = off[::every]
+    in_s = ot.in_tree.copy()
+    in_s[add] = 1
+    h0 = rng.gaussian_block(11, 3, g.n, r)
+    H = oracle.embed(og, ot, in_s, h0, 1, tol, maxit)
+    heat_ref, _ = oracle.heat(og, in_s, H)
+    with gpu_graph(g, rho) as (ctx, tree, _):
+        S = gpu.grass_sparsifier_create(ctx, tree)
+        try:
+            gpu.grass_sparsifier_add(ctx, S, dev(add.astype(np.int64)))
+            for P, dt, bound in ((gpu.GRASS_FP64, torch.float64, 1e-10), (gpu.GRASS_FP32, torch.float32, 1e-3)):
+                if P == gpu.GRASS_FP32 and maxit > 100:
+                    t2, m2 = 1e-6, 200
+                else:
+                    t2, m2 = tol, maxit
+                heat = torch.empty(heat_ref.shape[0], dtype=dt, device="cuda")
+                hm = gpu.grass_embed(ctx, S, dev(h0), r, 1, P, t2, m2, None, heat)
+                x = host(heat).astype(np.float64)
+                assert np.abs(x - heat_ref).max() <= bound * heat_ref.max(), P
+                assert hm == pytest.approx(heat_ref.max(), rel=bound)
+        finally:
+            gpu.grass_sparsifier_destroy(S)
+
+
+@pytest.mark.parametrize("added", [1, 126, 128, 129, 200])
+def test_rule_sides_agree(gpu, added):
+    """45 x 46 = 2070 vertices: up to 129 added edges take the core, more the
+    CG over all vertices; adding edges to S rebuilds it."""
+    import torch
+    g = graphs.grid2d_uniform(45, 46, seed=9)
+    og = oracle.from_graph(g)
+    ot = oracle.build_tree(og)
+    off = np.flatnonzero(ot.in_tree == 0)
+    h0 = rng.gaussian_block(12, 3, g.n, 4)
+    with gpu_graph(g) as (ctx, tree, _):
+        S = gpu.grass_sparsifier_create(ctx, tree)
+        try:
+            for part in (off[:max(1, added // 2)], off[:added]):
+                gpu.grass_sparsifier_add(ctx, S, dev(part.astype(np.int64)))
+                in_s = ot.in_tree.copy()
+                in_s[part] = 1
+                H = oracle.embed(og, ot, in_s, h0, 2, 1e-13, 2000)
+                heat_ref, _ = oracle.heat(og, in_s, H)
+                heat = torch.empty(heat_ref.shape[0], dtype=torch.float64, device="cuda")
+                gpu.grass_embed(ctx, S, dev(h0), 4, 2, gpu.GRASS_FP64, 1e-13, 2000, None, heat)
+                assert np.abs(host(heat) - heat_ref).max() <= 1e-10 * heat_ref.max()
+        finally:
+            gpu.grass_sparsifier_destroy(S)

@@ -50,12 +50,12 @@ def _graph(kind, n, seed):
 
 CASES = [("path", 2), ("path", 3), ("path", 3584), ("path", 3585), ("path", 20011),
          ("star", 700), ("star", 9001), ("star", 60013), ("heap", 4097), ("heap", 65535),
-         ("random", 3585), ("random", 7681), ("random", 300007), ("caterpillar", 12001),
+         ("random", 3585), ("random", 7681), ("random", 272300), ("random", 300007), ("caterpillar", 12001),
          ("brooms", 50021)]
 
 
 @pytest.mark.parametrize("kind,n", CASES)
-@pytest.mark.parametrize("r,prec", [(1, "fp64"), (2, "fp32"), (4, "fp64"), (16, "fp32"), (24, "fp32")])
+@pytest.mark.parametrize("r,prec", [(1, "fp64"), (2, "fp32"), (4, "fp64"), (8, "fp64"), (16, "fp32"), (24, "fp32"), (24, "fp64")])
 def test_unit_solve_matches_oracle(gpu, kind, n, r, prec):
     import torch
     g = _graph(kind, n, 7)
