@@ -284,6 +284,13 @@ grass_tree_t build_tree_impl(grass_ctx_t ctx, const grass_csr_t *A,
     T->ground = roots[0];
     T->g.nseg = (int64_t)roots.size();
     if (T->g.nseg > 1) T->g.seg_voff = voff;
+    // the graph's arrays, and the tour's of a tree that gets one, in one
+    // allocation; the temporaries from the context's arena
+    T->g.arena = &T->arena;
+    const int64_t mm = std::max<int64_t>(0, (A->nnz - A->n) / 2);
+    T->arena.chunk_min = (size_t)mm * 61 + (size_t)A->n * (A->n <= ctx->euler_max_n ? 104 : 25) + 65536;
+    ctx->build_tmp.reset();
+    ctx->build_tmp.chunk_min = (size_t)mm * 24 + (size_t)A->n * 180 + 65536;
     try {
         graph_extract(ctx, A, T->g);
         const int64_t n = T->g.n;
@@ -293,7 +300,7 @@ grass_tree_t build_tree_impl(grass_ctx_t ctx, const grass_csr_t *A,
         memset_d(ctx, T->isroot.p, 0, n);
         launch(ctx, k_mark_roots, cdiv(T->nroots, kBlock), kBlock, 0, T->nroots,
                (const int32_t *)T->roots.p, T->isroot.p);
-        T->in_tree.alloc(T->g.m);
+        T->in_tree.take(T->arena, T->g.m);
         if (user_eids) user_tree(ctx, T->g, user_eids, T->in_tree.p);
         else if (lsst_seed) lsst_build(ctx, T->g, *lsst_seed, T->in_tree.p, lsst_stats);
         else mst_boruvka(ctx, T->g, T->in_tree.p);
@@ -304,6 +311,7 @@ grass_tree_t build_tree_impl(grass_ctx_t ctx, const grass_csr_t *A,
         delete T;
         throw;
     }
+    if (ctx->build_tmp.bytes() > ((size_t)256 << 20)) ctx->build_tmp = Arena();
     return T;
 }
 

@@ -37,20 +37,26 @@ inline void check_cuda(cudaError_t e, const char *what) {
 
 // ---------------------------------------------------------------- buffers
 
-// Owning device buffer (synchronous cudaMalloc/cudaFree; long-lived data).
+struct Arena;
+
+// Device buffer: its own (synchronous cudaMalloc/cudaFree; long-lived data),
+// or carved from an arena that outlives it.
 template <typename T>
 struct DBuf {
     T *p = nullptr;
     size_t n = 0;
+    bool carved = false;
     DBuf() = default;
     DBuf(const DBuf &) = delete;
     DBuf &operator=(const DBuf &) = delete;
     ~DBuf() { release(); }
     void release() {
-        if (p) cudaFree(p);
+        if (p && !carved) cudaFree(p);
         p = nullptr;
         n = 0;
+        carved = false;
     }
+    void take(Arena &a, size_t count);
     void alloc(size_t count) {
         release();
         if (count == 0) count = 1;
@@ -108,6 +114,14 @@ struct Arena {
         a.n = count ? count : 1;
     }
 };
+
+template <typename T>
+void DBuf<T>::take(Arena &a, size_t count) {
+    release();
+    p = a.get<T>(count);
+    n = count ? count : 1;
+    carved = true;
+}
 
 // ---------------------------------------------------------------- context
 
@@ -168,9 +182,10 @@ struct grass_ctx_s {
     int lmax_amg = 0;           // 1: lambda_max estimates solve L_S by multigrid-preconditioned CG
     grass::Arena amg_tmp;       // the multigrid setup's temporary arrays
     grass::Arena core_tmp;      // the core form's
+    grass::Arena build_tmp;     // the tree construction's (kept up to 256 MB)
     int amg_fused = 1;          // 1: the multigrid PCG runs as one cooperative kernel (amg_fused.cu)
     int64_t amg_tail_n = 0;     // its levels of at most this many vertices run in one block
-    int64_t amg_warp_n = 16384; // its levels of at most this many vertices take a warp per row
+    int64_t amg_warp_n = 16384; // its levels of at most this many vertices take several lanes per row
     int64_t amg_warp_setup_n = 16384;   // hierarchy setup: levels of at most this many
                                         // vertices use the warp forms of the long-row kernels
     // a non-blocking stream of the context's own, on which multi-kernel
@@ -335,6 +350,7 @@ struct HeavyRows {
 
 struct GraphData {
     int64_t n = 0, m = 0;
+    Arena *arena = nullptr;           // the tree's: its arrays and the tour's
     DBuf<int32_t> adj_ptr;            // [n+1] off-diagonal adjacency in CSR order
     DBuf<int32_t> adj_col;            // [2m]
     DBuf<int32_t> adj_eid;            // [2m]
@@ -531,6 +547,7 @@ struct grass_tree_s {
     std::vector<int32_t> roots_h;
     grass::DBuf<int32_t> roots;        // [nroots]
     grass::DBuf<uint8_t> isroot;       // [n]
+    grass::Arena arena;               // one allocation for most of the arrays below
     grass::GraphData g;
     grass::DBuf<uint8_t> in_tree;     // [m]
     grass::TreeSchedule sched;         // elimination rounds (built on demand when units.built)

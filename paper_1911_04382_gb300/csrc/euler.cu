@@ -184,15 +184,16 @@ void euler_build(grass_ctx_t ctx, grass_tree_t T, const int32_t *tptr, const int
     const GraphData &g = T->g;
     const int64_t n = g.n, m = g.m, mt = L / 2;
     EulerTour &E = T->euler;
-    DBuf<int32_t> owner, es, eidx, nx0, nx1, d0, d1;
-    DBuf<int64_t> flag, pos;
-    owner.alloc(L);
-    es.alloc(L);
-    eidx.alloc(m);
+    Arena &tmp = ctx->build_tmp;
+    ASpan<int32_t> owner, es, eidx, nx0, nx1, d0, d1;
+    ASpan<int64_t> flag, pos;
+    tmp.get(owner, L);
+    tmp.get(es, L);
+    tmp.get(eidx, m);
     launch(ctx, k_eu_owner, cdiv(n, kBlock), kBlock, 0, n, tptr, owner.p);
     // dense tree-edge index: prefix positions of in_tree
-    flag.alloc(m + 1);
-    pos.alloc(m + 1);
+    tmp.get(flag, m + 1);
+    tmp.get(pos, m + 1);
     launch(ctx, k_u8_to_i64, cdiv(m, kBlock), kBlock, 0, m, (const uint8_t *)T->in_tree.p, flag.p);
     int64_t cnt = 0;
     scan_i64(ctx, flag.p, pos.p, m, &cnt);
@@ -201,10 +202,10 @@ void euler_build(grass_ctx_t ctx, grass_tree_t T, const int32_t *tptr, const int
            (const int64_t *)pos.p, eidx.p);
     launch(ctx, k_eu_edgeslots, cdiv(L, kBlock), kBlock, 0, L, (const int32_t *)owner.p, tocc, tsrc,
            es.p, (const int32_t *)eidx.p);
-    nx0.alloc(L);
-    nx1.alloc(L);
-    d0.alloc(L);
-    d1.alloc(L);
+    tmp.get(nx0, L);
+    tmp.get(nx1, L);
+    tmp.get(d0, L);
+    tmp.get(d1, L);
     launch(ctx, k_eu_succ, cdiv(L, kBlock), kBlock, 0, L, (const int32_t *)owner.p, tptr, tocc, tsrc,
            (const int32_t *)eidx.p, (const int32_t *)es.p, (const uint8_t *)T->isroot.p, nx0.p,
            d0.p);
@@ -217,49 +218,49 @@ void euler_build(grass_ctx_t ctx, grass_tree_t T, const int32_t *tptr, const int
         std::swap(d0.p, d1.p);
     }
     E.L = L;
-    E.tour.alloc(L);
-    E.ein.alloc(n);
-    E.eout.alloc(n);
-    E.par.alloc(n);
-    E.pw.alloc(n);
+    E.tour.take(T->arena, L);
+    E.ein.take(T->arena, n);
+    E.eout.take(T->arena, n);
+    E.par.take(T->arena, n);
+    E.pw.take(T->arena, n);
     launch(ctx, k_eu_final, cdiv(mt, kBlock), kBlock, 0, mt, (const int32_t *)es.p,
            (const int32_t *)owner.p, tocc, tsrc, (const int32_t *)d0.p,
            g.nseg > 1 ? (const int32_t *)g.seg_of.p : nullptr,
            g.nseg > 1 ? (const int64_t *)g.seg_voff_d.p : nullptr, (const double *)g.ew64.p,
            E.tour.p, E.ein.p, E.eout.p, E.par.p, E.pw.p);
-    E.head.alloc(L);
+    E.head.take(T->arena, L);
     memset_d(ctx, E.head.p, 0, L);
     launch(ctx, k_eu_roots, cdiv(T->nroots, kBlock), kBlock, 0, T->nroots,
            (const int32_t *)T->roots.p, g.nseg > 1 ? (const int64_t *)g.seg_voff_d.p : nullptr,
            E.ein.p, E.eout.p, E.pw.p, E.head.p);
-    E.ipw.alloc(n);
-    E.ipw32.alloc(n);
+    E.ipw.take(T->arena, n);
+    E.ipw32.take(T->arena, n);
     launch(ctx, k_eu_inv, cdiv(n, kBlock), kBlock, 0, n, (const double *)E.pw.p, E.ipw.p, E.ipw32.p);
     // preorder numbering and the tour / per-vertex arrays in it
     {
-        DBuf<int64_t> ent, epos;
-        ent.alloc(L + 1);
-        epos.alloc(L + 1);
+        ASpan<int64_t> ent, epos;
+        tmp.get(ent, L + 1);
+        tmp.get(epos, L + 1);
         launch(ctx, k_eu_isentry, cdiv(L, kBlock), kBlock, 0, L, (const int32_t *)E.tour.p, ent.p);
         int64_t ne = 0;
         scan_i64(ctx, ent.p, epos.p, L, &ne);
         if (ne != n - T->nroots) fail(GRASS_ERR_CUDA, "Euler tour: entry count mismatch");
-        E.pre.alloc(n);
-        E.vert.alloc(n);
+        E.pre.take(T->arena, n);
+        E.vert.take(T->arena, n);
         launch(ctx, k_eu_pre, cdiv(n, kBlock), kBlock, 0, n, (const int32_t *)E.ein.p,
                (const int64_t *)epos.p, g.nseg > 1 ? (const int32_t *)g.seg_of.p : nullptr,
                g.nseg > 1 ? (const int64_t *)g.seg_voff_d.p : nullptr, E.pre.p, E.vert.p);
-        E.tour_pre.alloc(L);
+        E.tour_pre.take(T->arena, L);
         launch(ctx, k_eu_tourpre, cdiv(L, kBlock), kBlock, 0, L, (const int32_t *)E.tour.p,
                (const int32_t *)E.pre.p, E.tour_pre.p);
-        E.head_pre.alloc(n);
+        E.head_pre.take(T->arena, n);
         memset_d(ctx, E.head_pre.p, 0, n);
         launch(ctx, k_eu_headpre, cdiv(T->nroots, kBlock), kBlock, 0, T->nroots,
                g.nseg > 1 ? (const int64_t *)g.seg_voff_d.p : nullptr, E.head_pre.p);
-        E.ein_pre.alloc(n);
-        E.eout_pre.alloc(n);
-        E.ipw_pre.alloc(n);
-        E.ipw32_pre.alloc(n);
+        E.ein_pre.take(T->arena, n);
+        E.eout_pre.take(T->arena, n);
+        E.ipw_pre.take(T->arena, n);
+        E.ipw32_pre.take(T->arena, n);
         launch(ctx, k_eu_prevals, cdiv(n, kBlock), kBlock, 0, n, (const int32_t *)E.vert.p,
                (const int32_t *)E.ein.p, (const int32_t *)E.eout.p, (const double *)E.ipw.p,
                (const float *)E.ipw32.p, E.ein_pre.p, E.eout_pre.p, E.ipw_pre.p, E.ipw32_pre.p);

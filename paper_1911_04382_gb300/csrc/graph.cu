@@ -156,9 +156,9 @@ void graph_extract(grass_ctx_t ctx, const grass_csr_t *A, GraphData &g) {
     memset_d(ctx, ctx->flags.p, 0, sizeof(int) * 4);
 
     g.n = n;
-    g.D64.alloc(n);
-    g.D32.alloc(n);
-    g.degG.alloc(n);
+    g.D64.take(*g.arena, n);
+    g.D32.take(*g.arena, n);
+    g.degG.take(*g.arena, n);
     int64_t *ucnt = ctx->scr<int64_t>(SCR_TMP0, n + 1);
     int64_t *acnt = ctx->scr<int64_t>(SCR_TMP1, n + 1);
     int64_t *ebase = ctx->scr<int64_t>(SCR_TMP2, n + 1);
@@ -172,18 +172,18 @@ void graph_extract(grass_ctx_t ctx, const grass_csr_t *A, GraphData &g) {
     if (na != 2 * m) fail(GRASS_ERR_INVALID, "off-diagonal pattern is not symmetric");
     if (m < n - g.nseg) fail(GRASS_ERR_DISCONNECTED, "fewer than n - (number of graphs) edges");
     g.m = m;
-    g.eu.alloc(m);
-    g.ev.alloc(m);
-    g.ew64.alloc(m);
-    g.ew32.alloc(m);
+    g.eu.take(*g.arena, m);
+    g.ev.take(*g.arena, m);
+    g.ew64.take(*g.arena, m);
+    g.ew32.take(*g.arena, m);
     int32_t *entry_eid = ctx->scr<int32_t>(SCR_Y, A->nnz + 1);
     launch(ctx, k_upper, cdiv(n, kBlock), kBlock, 0, n, A->rowptr, A->col, A->val,
            (const int64_t *)ebase, g.eu.p, g.ev.p, g.ew64.p, g.ew32.p, entry_eid);
-    g.adj_ptr.alloc(n + 1);
-    g.adj_col.alloc(2 * m);
-    g.adj_eid.alloc(2 * m);
-    g.adj_w64.alloc(2 * m);
-    g.adj_w32.alloc(2 * m);
+    g.adj_ptr.take(*g.arena, n + 1);
+    g.adj_col.take(*g.arena, 2 * m);
+    g.adj_eid.take(*g.arena, 2 * m);
+    g.adj_w64.take(*g.arena, 2 * m);
+    g.adj_w32.take(*g.arena, 2 * m);
     launch(ctx, k_adj, cdiv(n, kBlock), kBlock, 0, n, A->rowptr, A->col, A->val,
            (const int64_t *)aoff, (const int32_t *)entry_eid, g.adj_ptr.p, g.adj_col.p,
            g.adj_eid.p, g.adj_w64.p, g.adj_w32.p, ctx->flags.p);

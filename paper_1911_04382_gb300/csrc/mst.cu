@@ -118,18 +118,19 @@ void mst_boruvka(grass_ctx_t ctx, const GraphData &g, uint8_t *in_tree) {
 // doubles) in place of the graph's own.
 void mst_boruvka_w(grass_ctx_t ctx, const GraphData &g, const double *ew, uint8_t *in_tree) {
     const int64_t n = g.n, m = g.m;
-    DBuf<int32_t> comp, hook, nh, be, act0, act1;
-    DBuf<unsigned long long> bw;
-    DBuf<int64_t> flag, pos;
-    comp.alloc(n);
-    hook.alloc(n);
-    nh.alloc(n);
-    be.alloc(n);
-    bw.alloc(n);
-    act0.alloc(m);
-    act1.alloc(m);
-    flag.alloc(m + 1);
-    pos.alloc(m + 1);
+    Arena &tmp = ctx->build_tmp;
+    ASpan<int32_t> comp, hook, nh, be, act0, act1;
+    ASpan<unsigned long long> bw;
+    ASpan<int64_t> flag, pos;
+    tmp.get(comp, n);
+    tmp.get(hook, n);
+    tmp.get(nh, n);
+    tmp.get(be, n);
+    tmp.get(bw, n);
+    tmp.get(act0, m);
+    tmp.get(act1, m);
+    tmp.get(flag, m + 1);
+    tmp.get(pos, m + 1);
     unsigned int *nhooked = (unsigned int *)(ctx->flags.p + 1);
     int *changed = ctx->flags.p + 2;
     memset_d(ctx, in_tree, 0, (size_t)m);

@@ -1,5 +1,7 @@
-// tree.cu -- elimination schedule, numeric factorization and solves of the
-// spanning-tree matrix L_T (+ D).
+// tree.cu -- elimination rounds and their numeric factorization for the
+// spanning-tree matrix L_T (+ D).  A single tree with an Euler tour gets the
+// unit form instead (units.cu); its rounds are built only when their sizes
+// are asked for (grass_tree_info, grass_tree_schedule_info).
 //
 // Sec. III-H: a tree Laplacian factors in linear time.  The sequential
 // textbook order eliminates leaves first and needs as many dependent steps
@@ -301,30 +303,32 @@ static void schedule(grass_ctx_t ctx, grass_tree_t T, bool rounds) {
     const GraphData &g = T->g;
     const int64_t n = g.n;
     TreeSchedule &S = T->sched;
-    DBuf<int32_t> tptr, tocc, tsrc, elim_round;
-    DBuf<uint8_t> cls;
-    DBuf<int64_t> cnt, off;
-    DBuf<U64x2> val, voff;
-    tptr.alloc(n + 1);
-    cnt.alloc(n + 1);
-    off.alloc(n + 1);
+    Arena &tmp = ctx->build_tmp;
+    ASpan<int32_t> tptr, tocc, tsrc, elim_round;
+    ASpan<uint8_t> cls;
+    ASpan<int64_t> cnt, off;
+    ASpan<U64x2> val, voff;
+    tmp.reset();   // the spanning tree's temporaries are done with
+    tmp.get(tptr, n + 1);
+    tmp.get(cnt, n + 1);
+    tmp.get(off, n + 1);
     launch(ctx, k_tcount, cdiv(n, kBlock), kBlock, 0, n, g.adj_ptr.p, g.adj_eid.p,
            (const uint8_t *)T->in_tree.p, cnt.p);
     int64_t tslots = 0;
     scan_i64(ctx, cnt.p, off.p, n, &tslots);
     if (tslots != 2 * (n - T->nroots)) fail(GRASS_ERR_CUDA, "tree adjacency size mismatch");
-    tocc.alloc(tslots);
-    tsrc.alloc(tslots);
+    tmp.get(tocc, tslots);
+    tmp.get(tsrc, tslots);
     launch(ctx, k_tfill, cdiv(n, kBlock), kBlock, 0, n, g.adj_ptr.p, g.adj_col.p, g.adj_eid.p,
            (const uint8_t *)T->in_tree.p, (const int64_t *)off.p, tptr.p, tocc.p, tsrc.p);
     // the scan form pays off while its FP64 tour arrays stay near the L2
     // size; larger trees keep the elimination rounds only
     if (n <= ctx->euler_max_n && !T->euler.built) euler_build(ctx, T, tptr.p, tocc.p, tsrc.p, tslots);
     if (!rounds && unit_build(ctx, T, T->units)) return;
-    elim_round.alloc(n);
-    cls.alloc(n);
-    val.alloc(n + 1);
-    voff.alloc(n + 1);
+    tmp.get(elim_round, n);
+    tmp.get(cls, n);
+    tmp.get(val, n + 1);
+    tmp.get(voff, n + 1);
     S.n1.alloc(n);
     S.n2.alloc(n);
     S.src1.alloc(n);

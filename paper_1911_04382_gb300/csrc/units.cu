@@ -686,8 +686,7 @@ bool unit_build(grass_ctx_t ctx, grass_tree_t T, UnitTree &U) {
     U.built = false;
     if (!E.built || T->batch || T->nroots != 1 || ctx->num_sms <= 0 || n < 2) return false;
     U.arena.chunk_min = (size_t)n * 52 + ((size_t)1 << 20);
-    Arena tmp;
-    tmp.chunk_min = (size_t)n * 64 + ((size_t)1 << 20);
+    Arena &tmp = ctx->build_tmp;
     // preorder with the heavy child last
     auto *heavy = tmp.get<unsigned long long>(n);
     auto *shift = tmp.get<int64_t>(E.L + 1);
@@ -714,7 +713,6 @@ bool unit_build(grass_ctx_t ctx, grass_tree_t T, UnitTree &U) {
     int32_t *scnt = nullptr;
     int64_t n1 = 0;
     if (!unit_levels(ctx, n, parent, U.vid, nullptr, tmp, U, core, &scnt, &n1)) return false;
-    ctx->sync();   // the temporaries go
     return true;
 }
 
