@@ -201,7 +201,9 @@ def run_reference(args, w):
 # ---------------------------------------------------------------- kernel captures
 
 KERNEL_SOURCES = ["paper_1911_04382_gb300/csrc/krylov.cu", "paper_1911_04382_gb300/csrc/solve.cu",
+                  "paper_1911_04382_gb300/csrc/cg.cuh", "paper_1911_04382_gb300/csrc/core.cu",
                   "paper_1911_04382_gb300/csrc/tree_solve.cuh",
+                  "paper_1911_04382_gb300/csrc/units.cuh",
                   "paper_1911_04382_gb300/csrc/common.cuh",
                   "paper_1911_04382_gb300/csrc/amg_fused.cu"]
 
