@@ -125,12 +125,16 @@ void DBuf<T>::take(Arena &a, size_t count) {
 
 // ---------------------------------------------------------------- context
 
+// A slot that grows is freed and allocated anew, so a pointer to it is held
+// only across calls that do not use the slot.  The inner solves (SCR_CG_*,
+// SCR_CORE_*) run under the embedding, the estimates and the densification
+// rounds: what those hold lies in other slots.
 enum ScratchSlot {
     SCR_SCAN = 0, SCR_SCAN2, SCR_TMP0, SCR_TMP1, SCR_TMP2, SCR_TMP3,
     SCR_Y, SCR_H, SCR_CG_X, SCR_CG_R, SCR_CG_Z, SCR_CG_P, SCR_CG_Q,
     SCR_PCG_X, SCR_PCG_R, SCR_PCG_Z, SCR_PCG_P, SCR_PCG_Q, SCR_PCG_ZOLD, SCR_PCG_E,
     SCR_FILTER, SCR_FILTER2, SCR_HEAT, SCR_LMAX_V, SCR_LMAX_Y, SCR_PART2,
-    SCR_EU_S, SCR_EU_C, SCR_EU_P, SCR_EU_A, SCR_CG_XP,
+    SCR_EU_S, SCR_EU_C, SCR_EU_P, SCR_EU_A, SCR_CG_XP, SCR_CORE_D,
     SCR_SIM_V, SCR_SIM_E, SCR_SIM_C,
     SCR_PART_X, SCR_PART_Y, SCR_PART_1, SCR_AMG_Y, SCR_AMG_X, SCR_ONES,
     SCR_COUNT

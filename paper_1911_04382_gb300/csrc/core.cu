@@ -450,7 +450,7 @@ static void core_T(const CoreCall &c) {
     k.Y = (const T *)c.Y;
     k.X = (T *)c.X;
     k.F = ctx->scr<T>(SCR_CG_XP, (size_t)n * R);
-    k.dv = ctx->scr<T>(SCR_PCG_E, total);
+    k.dv = ctx->scr<T>(SCR_CORE_D, total);
     k.sptr = C.low.lv[0].sptr;
     k.vert = C.vert;
     k.maxbits = c.maxbits;

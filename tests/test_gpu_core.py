@@ -14,6 +14,7 @@ import pytest
 import oracle
 from synth import graphs, rng
 from tests.gpu_util import dev, gpu_graph, host
+from tests.test_gpu_parity import _densify_parity
 
 pytestmark = pytest.mark.gpu
 
@@ -87,3 +88,37 @@ def test_rule_sides_agree(gpu, added):
                 assert np.abs(host(heat) - heat_ref).max() <= 1e-10 * heat_ref.max()
         finally:
             gpu.grass_sparsifier_destroy(S)
+
+
+def _core_at_least(g, ot, in_s):
+    """A lower bound of the core's size: the vertices of the tree that rake and
+    compress leave when the ends of the added edges must stay (the ends and the
+    branchings of the paths between them; unit borders come on top)."""
+    added = np.flatnonzero((in_s != 0) & (ot.in_tree == 0))
+    og = oracle.from_graph(g)
+    pin = np.zeros(g.n, dtype=bool)
+    pin[og.eu[added]] = pin[og.ev[added]] = True
+    # paths that reach a vertex from below: 2 and more make it a branching
+    below = np.zeros(g.n, dtype=np.int64)
+    core = pin.copy()
+    for v in ot.order[::-1]:
+        core[v] |= below[v] >= 2
+        p = ot.parent[v]
+        if p >= 0 and (core[v] or below[v]):
+            below[p] += 1
+    return int(core.sum())
+
+
+def test_densify_core_larger_than_the_edge_list(gpu):
+    """Two FP64 rounds of 32 columns with a 5 % cap on a new context: round 2's
+    inner solves run on the core, whose block is larger than the list of
+    accepted edge ids that the rounds keep."""
+    g = graphs.grid2d_uniform(90, 80, seed=21)
+    cap, r = g.n // 20, 32
+    d, res = _densify_parity(gpu, g, 5.0, r, 2, 2, cap)
+    assert d["rounds"] == 2 and d["added_round"] == res.added
+    og = oracle.from_graph(g)
+    ot = oracle.build_tree(og)
+    in_s = ot.in_tree.copy()      # S in round 2
+    in_s[oracle.filter_edges(res.trace[0]["heat"], res.trace[0]["off"], res.theta[0], cap)] = 1
+    assert g.n >= 2048 and 16 * cap <= g.n and _core_at_least(g, ot, in_s) * r * 8 > 8 * (og.m + 1) + 256
