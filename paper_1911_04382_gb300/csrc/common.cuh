@@ -428,7 +428,7 @@ struct UnitFactor {
 // The sparsifier's core (core.cu): S's matrix with everything eliminated that
 // the vertices of its added edges leave hanging or in a chain.
 struct CoreForm {
-    bool built = false;             // tried for the present S; usable when low.built
+    bool usable = false;            // complete (else S has no core: tried, or no room)
     Arena arena;
     UnitTree low, tree;             // the elimination (one open level), the core's own tree
     UnitFactor low_f, tree_f;

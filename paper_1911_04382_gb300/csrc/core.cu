@@ -131,14 +131,11 @@ static bool core_wanted(const grass_sparsifier_s *S) {
     return T->units.built && n >= 2048 && added > 0 && 16 * added <= n;
 }
 
-static bool core_build(grass_ctx_t ctx, grass_sparsifier_t S) {
-    if (S->core && S->core->built) return S->core->low.built;
+// False: S keeps the CG over all vertices.
+static bool core_form(grass_ctx_t ctx, grass_sparsifier_t S, CoreForm &C) {
     grass_tree_t T = S->tree;
     const GraphData &g = T->g;
     const int64_t n = g.n, m = g.m, k = S->n_edges - (n - 1);
-    S->core = std::make_unique<CoreForm>();
-    CoreForm &C = *S->core;
-    C.built = true;
     Arena &tmp = ctx->core_tmp;
     tmp.reset();
     tmp.chunk_min = (size_t)m * 16 + (size_t)n * 48 + ((size_t)1 << 20);
@@ -161,10 +158,8 @@ static bool core_build(grass_ctx_t ctx, grass_sparsifier_t S) {
     int32_t *scnt = nullptr;
     int64_t n1 = 0;
     if (!unit_levels(ctx, n, parent, T->units.vid, pin, tmp, C.low, core, &scnt, &n1) ||
-        4 * n1 > n || n1 < 2) {
-        C.low.built = false;
+        4 * n1 > n || n1 < 2)
         return false;
-    }
     C.n = n1;
     C.nnz = 2 * (n1 - 1 + k);
     C.arena.chunk_min = (size_t)n1 * 96 + (size_t)k * 32 + ((size_t)1 << 20);
@@ -203,13 +198,29 @@ static bool core_build(grass_ctx_t ctx, grass_sparsifier_t S) {
     auto *core2 = tmp.get<int32_t>(n1);
     int32_t *scnt2 = nullptr;
     int64_t n2 = 0;
-    if (!unit_levels(ctx, n1, parent, nullptr, nullptr, tmp, C.tree, core2, &scnt2, &n2)) {
-        C.low.built = false;
+    if (!unit_levels(ctx, n1, parent, nullptr, nullptr, tmp, C.tree, core2, &scnt2, &n2))
         return false;
-    }
     unit_factor(ctx, C.tree, nullptr, C.tree_f);
     return true;
 }
+
+// S->core, once per change of S.  It is in place only when it is complete; a
+// tree that is not suited, or no room for the form, leaves an empty one (the
+// CG over all vertices needs none of its arrays), any other error none.
+static bool core_build(grass_ctx_t ctx, grass_sparsifier_t S) {
+    if (S->core) return S->core->usable;
+    auto C = std::make_unique<CoreForm>();
+    try {
+        C->usable = core_form(ctx, S, *C);
+    } catch (const Error &e) {
+        ctx->core_tmp = Arena();
+        if (e.st != GRASS_ERR_OOM) throw;
+    }
+    if (!C->usable) C = std::make_unique<CoreForm>();
+    S->core = std::move(C);
+    return S->core->usable;
+}
+
 
 // ---------------------------------------------------------------- solve
 

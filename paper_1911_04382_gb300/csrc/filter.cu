@@ -61,6 +61,7 @@ __global__ void k_s_fill(int64_t n, const int32_t *adj_ptr, const int32_t *adj_c
 void sparsifier_rebuild(grass_ctx_t ctx, grass_sparsifier_t S) {
     const GraphData &g = S->tree->g;
     const int64_t n = g.n, m = g.m;
+    S->core.reset();
     int64_t *flag = ctx->scr<int64_t>(SCR_TMP0, m + 1);
     int64_t *pos = ctx->scr<int64_t>(SCR_TMP1, m + 1);
     launch(ctx, k_off_flag, cdiv(m, kBlock), kBlock, 0, m, (const uint8_t *)S->in_s.p, flag);
@@ -98,7 +99,6 @@ void sparsifier_rebuild(grass_ctx_t ctx, grass_sparsifier_t S) {
         S->s_heavy.count = 0;
     }
     S->pre_ok = false;
-    S->core.reset();
     S->amg[0].reset();
     S->amg[1].reset();
 }

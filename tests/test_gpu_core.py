@@ -122,3 +122,85 @@ def test_densify_core_larger_than_the_edge_list(gpu):
     in_s = ot.in_tree.copy()      # S in round 2
     in_s[oracle.filter_edges(res.trace[0]["heat"], res.trace[0]["off"], res.theta[0], cap)] = 1
     assert g.n >= 2048 and 16 * cap <= g.n and _core_at_least(g, ot, in_s) * r * 8 > 8 * (og.m + 1) + 256
+
+
+def _on_core(gpu, ctx, S, n, h0, r, prec, maxit=16):
+    """Whether S's inner solves of `maxit` iterations run on its core, from the
+    algorithmic bytes of the kernel-family timing: an iteration over all
+    vertices moves at least 17 n-row blocks (the CG's vectors, the product's, the
+    tree solve's), one on the core a quarter of that at most (its rule)."""
+    gpu.grass_kernel_timing_enable(ctx, gpu.GRASS_KF_CG)
+    gpu.grass_embed(ctx, S, h0, r, 1, prec, 0.0, maxit)
+    _, launches, by = gpu.grass_kernel_timing_read(ctx)
+    gpu.grass_kernel_timing_enable(ctx, gpu.GRASS_KF_NONE)
+    blocks = by / (n * r * (8 if prec == gpu.GRASS_FP64 else 4)) / maxit
+    assert launches == 1 and (blocks >= 17 or blocks <= 10)
+    return blocks <= 10
+
+
+def _fill_device(torch, leave):
+    """Tensors that take the free device memory up to about `leave` bytes."""
+    held, size = [], torch.cuda.mem_get_info()[0] - leave
+    while size >= 1 << 21:
+        try:
+            held.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+        except torch.OutOfMemoryError:
+            size //= 2
+            continue
+        size = min(size, torch.cuda.mem_get_info()[0] - leave)
+    return held
+
+
+@pytest.mark.parametrize("leave_mb", [3, 6, 10])
+def test_core_without_room_serves_over_all_vertices(gpu, leave_mb):
+    """Device memory that ends somewhere in the core's construction (at least 13
+    MB here): the call is served by the CG over all vertices, the repeated one
+    too, and S has its core again once it has changed and there is room."""
+    import torch
+    g = graphs.grid2d_uniform(300, 301, seed=23)
+    og = oracle.from_graph(g)
+    ot = oracle.build_tree(og)
+    off = np.flatnonzero(ot.in_tree == 0)
+    h0 = rng.gaussian_block(13, 3, g.n, 2)
+    h0d, FP64 = dev(h0), gpu.GRASS_FP64
+    few, many = dev(off[::97].astype(np.int64)), dev(off[::5].astype(np.int64))
+    in_s = ot.in_tree.copy()
+    in_s[off[::97]] = 1
+    ref, _ = oracle.heat(og, in_s, oracle.embed(og, ot, in_s, h0, 1, 1e-13, 3000))
+    heat = torch.empty(ref.shape[0], dtype=torch.float64, device="cuda")
+    with gpu_graph(g) as (ctx, tree, _):
+        made = []
+
+        def sparsifier(ids):
+            S = gpu.grass_sparsifier_create(ctx, tree)
+            made.append(S)
+            gpu.grass_sparsifier_add(ctx, S, ids)
+            return S
+
+        def right(S):
+            heat.fill_(float("nan"))
+            gpu.grass_embed(ctx, S, h0d, 2, 1, FP64, 1e-13, 3000, None, heat)
+            assert np.abs(host(heat) - ref).max() <= 1e-10 * ref.max()
+
+        try:
+            # both forms' kernels, scratch and timing buffers first
+            assert _on_core(gpu, ctx, sparsifier(few), g.n, h0d, 2, FP64)
+            assert not _on_core(gpu, ctx, sparsifier(many), g.n, h0d, 2, FP64)
+            S = sparsifier(few)
+            host(heat.fill_(0.0))
+            torch.cuda.synchronize()
+            held = _fill_device(torch, leave_mb << 20)
+            try:
+                right(S)
+                right(S)
+                small = not _on_core(gpu, ctx, S, g.n, h0d, 2, FP64)
+            finally:
+                del held
+                torch.cuda.empty_cache()
+            assert small
+            right(S)
+            gpu.grass_sparsifier_add(ctx, S, dev(off[1:2].astype(np.int64)))
+            assert _on_core(gpu, ctx, S, g.n, h0d, 2, FP64)
+        finally:
+            for S in made:
+                gpu.grass_sparsifier_destroy(S)
