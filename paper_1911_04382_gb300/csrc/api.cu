@@ -290,7 +290,7 @@ grass_tree_t build_tree_impl(grass_ctx_t ctx, const grass_csr_t *A,
     const int64_t mm = std::max<int64_t>(0, (A->nnz - A->n) / 2);
     T->arena.chunk_min = (size_t)mm * 61 + (size_t)A->n * (A->n <= ctx->euler_max_n ? 104 : 25) + 65536;
     ctx->build_tmp.reset();
-    ctx->build_tmp.chunk_min = (size_t)mm * 24 + (size_t)A->n * 180 + 65536;
+    ctx->build_tmp.chunk_min = (size_t)mm * 24 + (size_t)A->n * (A->n <= ctx->euler_max_n ? 180 : 80) + 65536;
     try {
         graph_extract(ctx, A, T->g);
         const int64_t n = T->g.n;
@@ -311,7 +311,7 @@ grass_tree_t build_tree_impl(grass_ctx_t ctx, const grass_csr_t *A,
         delete T;
         throw;
     }
-    if (ctx->build_tmp.bytes() > ((size_t)256 << 20)) ctx->build_tmp = Arena();
+    trim(ctx->build_tmp);
     return T;
 }
 

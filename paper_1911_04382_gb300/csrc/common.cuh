@@ -123,6 +123,12 @@ void DBuf<T>::take(Arena &a, size_t count) {
     carved = true;
 }
 
+// What an idle arena of temporaries may keep for the next use.
+constexpr size_t kKeepTmp = (size_t)256 << 20;
+inline void trim(Arena &a) {
+    if (a.bytes() > kKeepTmp) a = Arena();
+}
+
 // ---------------------------------------------------------------- context
 
 // A slot that grows is freed and allocated anew, so a pointer to it is held
@@ -134,7 +140,7 @@ enum ScratchSlot {
     SCR_Y, SCR_H, SCR_CG_X, SCR_CG_R, SCR_CG_Z, SCR_CG_P, SCR_CG_Q,
     SCR_PCG_X, SCR_PCG_R, SCR_PCG_Z, SCR_PCG_P, SCR_PCG_Q, SCR_PCG_ZOLD, SCR_PCG_E,
     SCR_FILTER, SCR_FILTER2, SCR_HEAT, SCR_LMAX_V, SCR_LMAX_Y, SCR_PART2,
-    SCR_EU_S, SCR_EU_C, SCR_EU_P, SCR_EU_A, SCR_CG_XP, SCR_CORE_D,
+    SCR_EU_S, SCR_EU_C, SCR_EU_P, SCR_EU_A, SCR_CG_XP, SCR_CORE_D, SCR_CORE_E,
     SCR_SIM_V, SCR_SIM_E, SCR_SIM_C,
     SCR_PART_X, SCR_PART_Y, SCR_PART_1, SCR_AMG_Y, SCR_AMG_X, SCR_ONES,
     SCR_COUNT
@@ -185,8 +191,8 @@ struct grass_ctx_s {
     int amg_sweeps = 1;         // Jacobi sweeps before and after each coarse correction
     int lmax_amg = 0;           // 1: lambda_max estimates solve L_S by multigrid-preconditioned CG
     grass::Arena amg_tmp;       // the multigrid setup's temporary arrays
-    grass::Arena core_tmp;      // the core form's
-    grass::Arena build_tmp;     // the tree construction's (kept up to 256 MB)
+    grass::Arena core_tmp;      // the core form's (kept up to kKeepTmp)
+    grass::Arena build_tmp;     // the tree construction's (kept up to kKeepTmp)
     int amg_fused = 1;          // 1: the multigrid PCG runs as one cooperative kernel (amg_fused.cu)
     int64_t amg_tail_n = 0;     // its levels of at most this many vertices run in one block
     int64_t amg_warp_n = 16384; // its levels of at most this many vertices take several lanes per row
@@ -274,6 +280,13 @@ struct grass_ctx_s {
         return reinterpret_cast<T *>(b.p);
     }
     void sync() { GCK(cudaStreamSynchronize(stream)); }
+    // every buffer that calls have left behind for the next one
+    void give_back() {
+        for (auto &b : scratch) b.release();
+        amg_tmp = grass::Arena();
+        core_tmp = grass::Arena();
+        build_tmp = grass::Arena();
+    }
 };
 
 namespace grass {
@@ -402,7 +415,7 @@ struct UnitLevel {
     int32_t *ecore = nullptr;       // [nexp] next level's index of every export
     int32_t *epos = nullptr, *edst = nullptr;   // [nexp] its position there, its row in exp
     int32_t *sptr = nullptr;        // [n + 1] previous level's export rows by position
-    char *exp = nullptr, *V = nullptr;   // scratch: exports, level vector (32 FP64 columns)
+    char *exp = nullptr, *V = nullptr;   // scratch: exports (not of an open tree: the caller's), level vector (32 FP64 columns)
     double *dexp = nullptr, *w = nullptr;   // factor: load exports, weights to the parent
 };
 struct UnitTree {

@@ -138,9 +138,9 @@ static bool core_form(grass_ctx_t ctx, grass_sparsifier_t S, CoreForm &C) {
     const int64_t n = g.n, m = g.m, k = S->n_edges - (n - 1);
     Arena &tmp = ctx->core_tmp;
     tmp.reset();
-    tmp.chunk_min = (size_t)m * 16 + (size_t)n * 48 + ((size_t)1 << 20);
-    auto *flag = tmp.get<int64_t>(m + 1);
-    auto *at = tmp.get<int64_t>(m + 1);
+    tmp.chunk_min = (size_t)n * 36 + ((size_t)1 << 20);
+    auto *flag = ctx->scr<int64_t>(SCR_TMP0, m + 1);
+    auto *at = ctx->scr<int64_t>(SCR_TMP1, m + 1);
     auto *xu = tmp.get<int32_t>(k), *xv = tmp.get<int32_t>(k);
     auto *xw = tmp.get<double>(k);
     auto *pin = tmp.get<uint8_t>(n);
@@ -154,7 +154,7 @@ static bool core_form(grass_ctx_t ctx, grass_sparsifier_t S, CoreForm &C) {
            (const int32_t *)g.ev.p, (const double *)g.ew64.p, (const int32_t *)T->units.pos, xu, xv,
            xw, pin);
     copy_d(ctx, parent, T->units.parent, n * sizeof(int32_t));
-    C.low.arena.chunk_min = (size_t)n * 40 + ((size_t)1 << 20);
+    C.low.arena.chunk_min = (size_t)n * 32 + ((size_t)1 << 20);
     int32_t *scnt = nullptr;
     int64_t n1 = 0;
     if (!unit_levels(ctx, n, parent, T->units.vid, pin, tmp, C.low, core, &scnt, &n1) ||
@@ -162,7 +162,7 @@ static bool core_form(grass_ctx_t ctx, grass_sparsifier_t S, CoreForm &C) {
         return false;
     C.n = n1;
     C.nnz = 2 * (n1 - 1 + k);
-    C.arena.chunk_min = (size_t)n1 * 96 + (size_t)k * 32 + ((size_t)1 << 20);
+    C.arena.chunk_min = (size_t)n1 * 56 + (size_t)k * 32 + ((size_t)1 << 19);
     UnitLevel &L = C.low.lv[0];
     L.sptr = C.arena.get<int32_t>(n1 + 1);
     unit_group(ctx, C.low, L, n1, nullptr, scnt, tmp, L.sptr);
@@ -217,6 +217,7 @@ static bool core_build(grass_ctx_t ctx, grass_sparsifier_t S) {
         if (e.st != GRASS_ERR_OOM) throw;
     }
     if (!C->usable) C = std::make_unique<CoreForm>();
+    trim(ctx->core_tmp);
     S->core = std::move(C);
     return S->core->usable;
 }
@@ -458,6 +459,7 @@ static void core_T(const CoreCall &c) {
     std::memset((void *)&k, 0, sizeof(k));
     k.low = unit_args<T, R>(C.low, C.low_f, &smem_low);
     smem = std::max(smem, smem_low);
+    k.low.lv[0].exp = ctx->scr<T>(SCR_CORE_E, (size_t)C.low.lv[0].nexp * R);
     k.Y = (const T *)c.Y;
     k.X = (T *)c.X;
     k.F = ctx->scr<T>(SCR_CG_XP, (size_t)n * R);

@@ -83,12 +83,15 @@ using namespace grass;
 // h0, v0, b, x) plus what the library allocates for the tree, the
 // sparsifier, the embedding blocks and the Krylov vectors.  The per-vertex,
 // per-nonzero and per-column terms are upper bounds of the library's
-// allocations (checked against measured use by the tests).
+// allocations (checked against measured use by the tests).  Per edge (half a
+// nonzero) up to 142 bytes: graph 61, sparsifier's edge list 25, flags,
+// positions, heats and ids of the rounds 56; per column 48: two embedding
+// blocks and four CG vectors in FP64.
 extern "C" int64_t grass_server_footprint(int64_t n, int64_t nnz, int r, int rounds) {
     if (n <= 0 || nnz < 0 || r <= 0 || rounds <= 0) return -1;
     const int64_t inputs = 8 * (n + 1) + 12 * nnz + 8 * n * r * (int64_t)rounds +
                            8 * n * (int64_t)rounds + 16 * n;
-    const int64_t library = 600 * n + 40 * nnz + 48 * n * (int64_t)r;
+    const int64_t library = 500 * n + 72 * nnz + 48 * n * (int64_t)r;
     return inputs + library + (64LL << 20);
 }
 
@@ -119,9 +122,12 @@ void grass_server_s::run(int slot, grass_ctx_t ctx, Ticket &t) {
     grass_tree_t tree = nullptr;
     grass_sparsifier_t S = nullptr;
     grass_status st = grass_build_tree(ctx, &A, 0, &tree);
+    ctx->build_tmp = Arena();   // nothing below builds a tree
     const double t_tree = now();
     if (st == GRASS_OK) st = grass_densify(ctx, tree, &q.params, (const double *)h0.p,
                                            (const double *)v0.p, &S, &res.sparsify);
+    if (S) S->core.reset();     // one column with D: the PCG takes no core
+    ctx->core_tmp = Arena();
     const double t_dens = now();
     if (st == GRASS_OK) {
         st = grass_pcg_solve(ctx, S, (const double *)b.p, (double *)x.p, q.tol, q.maxit,
@@ -138,7 +144,7 @@ void grass_server_s::run(int slot, grass_ctx_t ctx, Ticket &t) {
     if (tree) grass_tree_destroy(tree);
     // scratch grows with the largest request a context has served: give it
     // back so the budget accounts for this request alone
-    for (auto &sc : ctx->scratch) sc.release();
+    ctx->give_back();
     res.ms_h2d = 1e3 * (t_in - res.t_admit);
     res.ms_tree = 1e3 * (t_tree - t_in);
     res.ms_densify = 1e3 * (t_dens - t_tree);
@@ -180,7 +186,7 @@ void grass_server_s::worker(int slot) {
                 run(slot, ctx, *t);
             } catch (const Error &e) {
                 set_error(t->res, e.st, e.msg.c_str());
-                for (auto &sc : ctx->scratch) sc.release();
+                ctx->give_back();
             } catch (...) {
                 set_error(t->res, GRASS_ERR_CUDA, "unexpected internal error");
             }

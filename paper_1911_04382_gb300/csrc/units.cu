@@ -653,7 +653,7 @@ bool unit_levels(grass_ctx_t ctx, int64_t n, int32_t *parent, const int32_t *vid
         if (n1 > nl / 2 ||
             UnitSmem<double>::lists(L.local, L.elim) + UnitSmem<double>::rows(L.local, 8) > kTailSmem)
             return false;
-        L.exp = U.arena.get<char>((size_t)L.nexp * 32 * sizeof(double));
+        if (!U.open) L.exp = U.arena.get<char>((size_t)L.nexp * 32 * sizeof(double));
         L.dexp = U.arena.get<double>(L.nexp);
         L.ecore = U.arena.get<int32_t>(L.nexp);
         scnt = tmp.get<int32_t>(n1);
