@@ -313,13 +313,20 @@ grass_status grass_build_lsst(grass_ctx_t ctx, const grass_csr_t *A, uint64_t se
  * (a forest, or no Euler tour), OOM, CUDA. */
 grass_status grass_tree_stretch(grass_ctx_t ctx, grass_tree_t tree, double *stretch, double *total);
 
-/* Sizes: n, m (edges), factor_rounds (contraction rounds of the tree
- * elimination schedule).  Any pointer may be NULL.  Host outputs. */
+/* Sizes: n, m (edges), factor_rounds (contraction rounds of the tree's
+ * elimination schedule).  Any pointer may be NULL.  Host outputs.
+ * n and m are at hand.  A single tree of at most euler_max_n vertices solves
+ * in units and keeps no schedule: the first call that asks for factor_rounds
+ * (or for grass_tree_schedule_info) contracts the tree once on the context's
+ * stream, a few ms at a million vertices with about 130 bytes a vertex of
+ * device memory meanwhile, and may return OOM, CUDA; the sizes then stay on
+ * the host.  The solves do not change. */
 grass_status grass_tree_info(grass_tree_t tree, int64_t *n, int64_t *m, int64_t *factor_rounds);
 
 /* Per-round sizes of the elimination schedule (host outputs, room for cap
  * rounds each, any may be NULL): vertices eliminated, vertices receiving
- * updates, and updates (contributions), round by round. */
+ * updates, and updates (contributions), round by round.  First call on a
+ * tree: see grass_tree_info. */
 grass_status grass_tree_schedule_info(grass_tree_t tree, int64_t *eliminated, int64_t *receivers,
                                       int64_t *contributions, int64_t cap);
 

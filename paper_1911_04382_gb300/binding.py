@@ -361,9 +361,12 @@ def grass_tree_destroy(tree: int) -> None:
     lib().grass_tree_destroy(tree)
 
 
-def grass_tree_info(tree: int) -> tuple[int, int, int]:
-    n, m, r = _i64(), _i64(), _i64()
-    _check(None, lib().grass_tree_info(tree, C.byref(n), C.byref(m), C.byref(r)), "grass_tree_info")
+def grass_tree_info(tree: int, rounds: bool = True) -> tuple[int, int, int]:
+    """(n, m, contraction rounds); rounds=False leaves the last one out (0),
+    whose first query may have to contract the tree."""
+    n, m, r = _i64(), _i64(), _i64(0)
+    _check(None, lib().grass_tree_info(tree, C.byref(n), C.byref(m), C.byref(r) if rounds else None),
+           "grass_tree_info")
     return n.value, m.value, r.value
 
 

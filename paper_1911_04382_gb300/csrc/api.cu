@@ -289,6 +289,7 @@ grass_tree_t build_tree_impl(grass_ctx_t ctx, const grass_csr_t *A,
     T->g.arena = &T->arena;
     const int64_t mm = std::max<int64_t>(0, (A->nnz - A->n) / 2);
     T->arena.chunk_min = (size_t)mm * 61 + (size_t)A->n * (A->n <= ctx->euler_max_n ? 104 : 25) + 65536;
+    TrimLater later{ctx->build_tmp};
     ctx->build_tmp.reset();
     ctx->build_tmp.chunk_min = (size_t)mm * 24 + (size_t)A->n * (A->n <= ctx->euler_max_n ? 180 : 80) + 65536;
     try {
@@ -311,7 +312,6 @@ grass_tree_t build_tree_impl(grass_ctx_t ctx, const grass_csr_t *A,
         delete T;
         throw;
     }
-    trim(ctx->build_tmp);
     return T;
 }
 
@@ -466,18 +466,7 @@ grass_status grass_tree_schedule_info(grass_tree_t T, int64_t *eliminated, int64
     for (int k = 0; k < S.rounds && k < cap; ++k) {
         if (eliminated) eliminated[k] = S.elim_off[k + 1] - S.elim_off[k];
         if (receivers) receivers[k] = S.rcv_off[k + 1] - S.rcv_off[k];
-        if (contributions) {
-            contributions[k] = 0;   // filled below from the host offsets
-        }
-    }
-    if (contributions) {
-        // contributions of round k = rcv_beg[rcv_off[k+1]] - rcv_beg[rcv_off[k]]
-        std::vector<int32_t> beg(S.n_rcv + 1);
-        if (cudaMemcpy(beg.data(), S.rcv_beg.p, beg.size() * sizeof(int32_t),
-                       cudaMemcpyDeviceToHost) != cudaSuccess)
-            return GRASS_ERR_CUDA;
-        for (int k = 0; k < S.rounds && k < cap; ++k)
-            contributions[k] = beg[S.rcv_off[k + 1]] - beg[S.rcv_off[k]];
+        if (contributions) contributions[k] = S.contrib_off[k + 1] - S.contrib_off[k];
     }
     API_END
 }

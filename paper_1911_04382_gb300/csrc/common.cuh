@@ -128,6 +128,11 @@ constexpr size_t kKeepTmp = (size_t)256 << 20;
 inline void trim(Arena &a) {
     if (a.bytes() > kKeepTmp) a = Arena();
 }
+// trims when the use of an arena ends, by an error too
+struct TrimLater {
+    Arena &a;
+    ~TrimLater() { trim(a); }
+};
 
 // ---------------------------------------------------------------- context
 
@@ -651,8 +656,9 @@ void tree_schedule(grass_ctx_t ctx, grass_tree_t T);
 // every slot in tsrc; L slots), before the contraction rounds modify it.
 void euler_build(grass_ctx_t ctx, grass_tree_t T, const int32_t *tptr, const int32_t *tocc,
                  const int32_t *tsrc, int64_t L);
-// The elimination rounds of a tree that has the unit form (their sizes are
-// reported by the API; its solves do not use them).
+// The sizes of the elimination rounds of a tree that has the unit form (the
+// API reports them; its solves do not use the rounds): contracted once, on
+// demand, and kept on the host.
 void tree_rounds(grass_ctx_t ctx, grass_tree_t T);
 void tree_factor(grass_ctx_t ctx, grass_tree_t T, bool with_D, TreeFactor &f);
 // Algorithmic bytes of one tree solve of r columns of s bytes.

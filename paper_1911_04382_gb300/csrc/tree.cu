@@ -284,12 +284,6 @@ static void tree_pack(grass_ctx_t ctx, grass_tree_t T) {
            (const int4 *)S.fwd_rec.p + r0, (const int32_t *)locmap.p, S.fwd_loc.p);
     launch(ctx, k_tail_bwd, cdiv(ne - e0, kBlock), kBlock, 0, ne - e0,
            (const int4 *)S.bwd_rec.p + e0, (const int32_t *)locmap.p, S.bwd_loc.p);
-    DBuf<int64_t> coff;
-    coff.alloc(S.rounds + 1);
-    launch(ctx, k_round_contrib, cdiv(S.rounds + 1, kBlock), kBlock, 0, (int64_t)S.rounds + 1,
-           (const int64_t *)S.d_offs.p, (const int32_t *)S.rcv_beg.p, coff.p);
-    S.contrib_off.assign(S.rounds + 1, 0);
-    d2h(ctx, S.contrib_off.data(), coff.p, (S.rounds + 1) * sizeof(int64_t));
     const int64_t c0 = S.contrib_off[k0];
     S.tail_c0 = c0;
     S.contrib_loc.alloc(S.n_contrib - c0);
@@ -298,11 +292,11 @@ static void tree_pack(grass_ctx_t ctx, grass_tree_t T) {
     ctx->sync();
 }
 
-// rounds: build the elimination rounds even when the tree has the unit form
-static void schedule(grass_ctx_t ctx, grass_tree_t T, bool rounds) {
+// The rounds into S.  sizes: their sizes alone are wanted, of a tree that has
+// the unit form; else the solve's records too, unless the tree gets that form.
+static void schedule(grass_ctx_t ctx, grass_tree_t T, TreeSchedule &S, bool sizes) {
     const GraphData &g = T->g;
     const int64_t n = g.n;
-    TreeSchedule &S = T->sched;
     Arena &tmp = ctx->build_tmp;
     ASpan<int32_t> tptr, tocc, tsrc, elim_round;
     ASpan<uint8_t> cls;
@@ -323,8 +317,8 @@ static void schedule(grass_ctx_t ctx, grass_tree_t T, bool rounds) {
            (const uint8_t *)T->in_tree.p, (const int64_t *)off.p, tptr.p, tocc.p, tsrc.p);
     // the scan form pays off while its FP64 tour arrays stay near the L2
     // size; larger trees keep the elimination rounds only
-    if (n <= ctx->euler_max_n && !T->euler.built) euler_build(ctx, T, tptr.p, tocc.p, tsrc.p, tslots);
-    if (!rounds && unit_build(ctx, T, T->units)) return;
+    if (!sizes && n <= ctx->euler_max_n) euler_build(ctx, T, tptr.p, tocc.p, tsrc.p, tslots);
+    if (!sizes && unit_build(ctx, T, T->units)) return;
     tmp.get(elim_round, n);
     tmp.get(cls, n);
     tmp.get(val, n + 1);
@@ -387,13 +381,26 @@ static void schedule(grass_ctx_t ctx, grass_tree_t T, bool rounds) {
     }
     S.d_offs.alloc(h.size());
     h2d(ctx, S.d_offs.p, h.data(), h.size() * sizeof(int64_t));
-    tree_pack(ctx, T);
+    auto *coff = tmp.get<int64_t>(S.rounds + 1);
+    launch(ctx, k_round_contrib, cdiv(S.rounds + 1, kBlock), kBlock, 0, (int64_t)S.rounds + 1,
+           (const int64_t *)S.d_offs.p, (const int32_t *)S.rcv_beg.p, coff);
+    S.contrib_off.assign(S.rounds + 1, 0);
+    d2h(ctx, S.contrib_off.data(), coff, (S.rounds + 1) * sizeof(int64_t));
+    if (!sizes) tree_pack(ctx, T);
 }
 
-void tree_schedule(grass_ctx_t ctx, grass_tree_t T) { schedule(ctx, T, false); }
+void tree_schedule(grass_ctx_t ctx, grass_tree_t T) { schedule(ctx, T, T->sched, false); }
 
 void tree_rounds(grass_ctx_t ctx, grass_tree_t T) {
-    if (T->sched.rounds == 0) schedule(ctx, T, true);
+    if (T->sched.rounds > 0) return;
+    TrimLater later{ctx->build_tmp};
+    ctx->build_tmp.chunk_min = (size_t)T->g.n * 80 + 65536;
+    TreeSchedule S;   // its device arrays go with it
+    schedule(ctx, T, S, true);
+    T->sched.elim_off = std::move(S.elim_off);
+    T->sched.rcv_off = std::move(S.rcv_off);
+    T->sched.contrib_off = std::move(S.contrib_off);
+    T->sched.rounds = S.rounds;
 }
 
 double tree_solve_bytes(const grass_tree_s *T, int r, double s) {

@@ -89,3 +89,31 @@ def test_unit_solve_matches_oracle(gpu, kind, n, r, prec):
             scan = r == 1 and not with_D      # the scan form's block sums follow the launch shape
             assert scan or torch.equal(odd, X), with_D
             odd.copy_(Bd)
+
+
+@pytest.mark.parametrize("n", [3, 3585, 20011])
+def test_round_sizes_on_demand(gpu, n):
+    """The elimination rounds' sizes of a tree that solves in units: those of
+    the same tree as a batch of one, and after the query the tree solves as
+    before it and holds no more device memory."""
+    import torch
+    g = _graph("random", n, 8)
+    B = dev(rng.gaussian_block(5, 7, n, 4))
+    X, Y = torch.empty_like(B), torch.empty_like(B)
+    with gpu_graph(g, 0) as (ctx, tree, csr):
+        forest = gpu.grass_build_forest(ctx, *csr, [0, n])
+        try:
+            sizes = gpu.grass_tree_schedule_info(forest)
+            assert gpu.grass_tree_info(forest) == (n, n - 1, len(sizes[0])) and sum(sizes[0]) == n - 1
+        finally:
+            gpu.grass_tree_destroy(forest)
+        assert gpu.grass_tree_info(tree, rounds=False)[:2] == (n, n - 1)
+        gpu.grass_tree_solve(ctx, tree, 1, 4, gpu.GRASS_FP64, B, X)
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        assert gpu.grass_tree_schedule_info(tree) == sizes
+        assert gpu.grass_tree_info(tree) == (n, n - 1, len(sizes[0]))
+        torch.cuda.synchronize()
+        assert torch.cuda.mem_get_info()[0] == free
+        gpu.grass_tree_solve(ctx, tree, 1, 4, gpu.GRASS_FP64, B, Y)
+        assert torch.equal(X, Y)
