@@ -147,7 +147,9 @@ grass_status grass_ctx_set_wait_limit(grass_ctx_t ctx, int64_t polls, int hold_b
  *                         form with one column use at most 512 of them
  *   "tree_tail_items"     rounds at the end whose total work is below this
  *                         many items run in one block (work: surviving
- *                         vertices x max(1, r/4); default 2048; 0 = none)
+ *                         vertices x max(1, r/4); default 2048; 0 = none);
+ *                         for the solves in elimination rounds (forests, trees
+ *                         of more than euler_max_n vertices)
  *   "euler_solve"         1 (default): grounded solves of L_T alone (no D)
  *                         with one column use the scan form (two segmented
  *                         prefix sums: along the Euler tour for a solve on
@@ -579,7 +581,8 @@ grass_status grass_pcg_solve_batch(grass_ctx_t ctx, grass_sparsifier_t S, const 
 /* Autotuner (no counterpart in the paper): time the tree (forest) solve of
  * r columns under each launch shape -- threads per block {256, 512, 1024},
  * blocks per SM {1, 2, 4}, shared-memory tail {1024, 4096, 16384} items --
- * and keep the fastest on ctx (as grass_ctx_set_param would).  best: host
+ * and keep the fastest on ctx (as grass_ctx_set_param would).  The tail is
+ * left as it is when the timed solve has none (see "tree_tail_items").  best: host
  * [3] = threads, blocks per SM, tail items; best_ms: host, its time per
  * solve.  Results of every solve are the same under any shape. */
 grass_status grass_autotune(grass_ctx_t ctx, grass_tree_t tree, int r, grass_prec prec,

@@ -906,7 +906,9 @@ extern "C" grass_status grass_pcg_solve_batch(grass_ctx_t ctx, grass_sparsifier_
 // Times the tree (forest) solve of `tree` for r columns under every launch
 // shape below and keeps the fastest on the context: threads per block,
 // blocks per SM, and the tail size (how many final rounds run in one block
-// from shared memory).  The solve's results do not depend on the shape.
+// from shared memory).  A solve in units or in the scan form has no tail: its
+// shapes leave the context's value as it is.  The solve's results do not depend
+// on the shape.
 
 extern "C" grass_status grass_autotune(grass_ctx_t ctx, grass_tree_t T, int r, grass_prec prec,
                                        int64_t *best, double *best_ms) {
@@ -922,9 +924,11 @@ extern "C" grass_status grass_autotune(grass_ctx_t ctx, grass_tree_t T, int r, g
     memset_d(ctx, Y.p, 0, n * r * es);
     const int threads[] = {256, 512, 1024};
     const int bpsm[] = {1, 2, 4};
-    const int64_t tails[] = {1024, 4096, 16384};
     const int keep_t = ctx->tree_threads, keep_b = ctx->tree_bpsm;
     const int64_t keep_tail = ctx->tree_tail_items;
+    const bool tail = !T->units.built && !(r == 1 && ctx->euler_solve && T->euler.built);
+    const std::vector<int64_t> tails =
+        tail ? std::vector<int64_t>{1024, 4096, 16384} : std::vector<int64_t>{keep_tail};
     cudaEvent_t e0, e1;
     GCK(cudaEventCreate(&e0));
     GCK(cudaEventCreate(&e1));

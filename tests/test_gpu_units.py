@@ -117,3 +117,14 @@ def test_round_sizes_on_demand(gpu, n):
         assert torch.cuda.mem_get_info()[0] == free
         gpu.grass_tree_solve(ctx, tree, 1, 4, gpu.GRASS_FP64, B, Y)
         assert torch.equal(X, Y)
+
+
+def test_autotune_leaves_the_tail_of_a_tree_without_one(gpu):
+    """A single tree's solve has no tail to tune: the forests' setting stays."""
+    g = _graph("random", 7681, 8)
+    with gpu_graph(g, 0) as (ctx, tree, _):
+        for tail in (777, 20000):
+            gpu.grass_ctx_set_param(ctx, "tree_tail_items", tail)
+            for r in (1, 8):
+                best, ms = gpu.grass_autotune(ctx, tree, r, gpu.GRASS_FP32)
+                assert best[2] == tail and best[0] in (256, 512, 1024) and ms > 0
