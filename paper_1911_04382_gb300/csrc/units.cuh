@@ -591,7 +591,10 @@ __device__ __forceinline__ bool unit_solve_dev(const UnitArgs<T> &a, unsigned in
             unit_coef(g, L, u, m, s);
             cp_async_commit();
         }
-        if (!grid_sync(bar, budget, err, epoch)) return false;
+        if (!grid_sync(bar, budget, err, epoch)) {
+            cp_async_wait<0>();   // the block ends with none of its copies in flight
+            return false;
+        }
         for (int t = last; t >= 0; t -= GG) {
             const int u = t / parts, cg0 = (t % parts) * span;
             const int4 m = L.meta[u];
