@@ -97,7 +97,8 @@ static int64_t power_steps_until(grass_ctx_t ctx, grass_sparsifier_t S, const do
         lap_mm(ctx, r, prec, n, 2 * g.m, g.adj_ptr.p, g.adj_col.p, w, nullptr, H, Y,
                prev >= 0 ? maxslot(ctx, prev) : nullptr, GRASS_KF_SPMM_G, &g.heavy);
         memset_d(ctx, maxslot(ctx, cur), 0, sizeof(unsigned long long));
-        inner += s_solve(ctx, S, false, r, prec, Y, H, inner_tol, inner_maxit, maxslot(ctx, cur));
+        inner += s_solve(ctx, S, false, r, prec, Y, H, inner_tol, inner_maxit, maxslot(ctx, cur),
+                         (int64_t)t * inner_maxit);
         prev = cur;
         cur ^= 1;
         if (stop_when_capped && !S->is_tree && s + 1 < t) {

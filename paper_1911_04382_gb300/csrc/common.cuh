@@ -686,9 +686,10 @@ void unit_factor(grass_ctx_t ctx, const UnitTree &U, const double *D, UnitFactor
 // ---------------------------------------------------------------- core.cu
 
 // X = L_S^{-1} Y (grounded) by CG on the core; false when S has no core form
-// (the caller takes the CG over all vertices).  Arguments as s_solve.
+// (the caller takes the CG over all vertices) or its build would not pay in
+// `its` iterations.  Arguments as s_solve.
 bool core_solve(grass_ctx_t ctx, grass_sparsifier_t S, int r, grass_prec prec, const void *Y, void *X,
-                double tol, int maxit, unsigned long long *maxbits);
+                double tol, int maxit, unsigned long long *maxbits, int64_t its);
 
 // In-place tree solve of the n x r block Y (prec), or from B into Y;
 // optionally tracks the max |x| bit pattern into maxbits (device, uint64 for
@@ -728,9 +729,11 @@ void max_abs_bits(grass_ctx_t ctx, grass_prec prec, int64_t count, const void *X
 // X = L_S^{-1} Y (grounded, or (L_S + D)^{-1} Y when with_D), r columns, by
 // the tree solve (S is the tree) or tree-preconditioned CG.  Y is preserved
 // unless S is the tree (then Y may be X).  Returns inner iterations (max over
-// columns).  maxbits: optional max|X| tracking.
+// columns).  maxbits: optional max|X| tracking.  its: the iterations that the
+// call this solve is part of allows on S in all (0: maxit).
 int64_t s_solve(grass_ctx_t ctx, grass_sparsifier_t S, bool with_D, int r, grass_prec prec,
-                const void *Y, void *X, double tol, int maxit, unsigned long long *maxbits);
+                const void *Y, void *X, double tol, int maxit, unsigned long long *maxbits,
+                int64_t its = 0);
 
 void pcg_solve(grass_ctx_t ctx, grass_sparsifier_t S, const double *b, double *x, double tol,
                int maxit, grass_prec prec, double refine_tol, double inner_tol, int inner_maxit,

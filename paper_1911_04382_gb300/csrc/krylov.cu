@@ -290,7 +290,8 @@ __global__ void k_note_solve(double *acc, double its, double capped) {
 }
 
 int64_t s_solve(grass_ctx_t ctx, grass_sparsifier_t S, bool with_D, int r, grass_prec prec,
-                const void *Y, void *X, double tol, int maxit, unsigned long long *maxbits) {
+                const void *Y, void *X, double tol, int maxit, unsigned long long *maxbits,
+                int64_t its) {
     grass_tree_t T = S->tree;
     const GraphData &g = T->g;
     const int64_t n = g.n, total = n * r;
@@ -319,7 +320,9 @@ int64_t s_solve(grass_ctx_t ctx, grass_sparsifier_t S, bool with_D, int r, grass
     }
     if (ctx->num_sms > 0) {
         // one column stays with the scan form's float-pair sums
-        if (!with_D && r > 1 && core_solve(ctx, S, r, prec, Y, X, tol, maxit, maxbits)) return 0;
+        if (!with_D && r > 1 && core_solve(ctx, S, r, prec, Y, X, tol, maxit, maxbits,
+                                         its > 0 ? its : maxit))
+            return 0;
         CGCall call{ctx, S, with_D, prec, Y, X, tol, maxit, maxbits};
         GRASS_DISPATCH_R(r, cg_R, call);
         return 0;

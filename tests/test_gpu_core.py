@@ -124,17 +124,18 @@ def test_densify_core_larger_than_the_edge_list(gpu):
     assert g.n >= 2048 and 16 * cap <= g.n and _core_at_least(g, ot, in_s) * r * 8 > 8 * (og.m + 1) + 256
 
 
-def _on_core(gpu, ctx, S, n, h0, r, prec, maxit=16):
+def _on_core(gpu, ctx, S, n, h0, r, prec, maxit=160, t=1):
     """Whether S's inner solves of `maxit` iterations run on its core, from the
     algorithmic bytes of the kernel-family timing: an iteration over all
-    vertices moves at least 17 n-row blocks (the CG's vectors, the product's, the
-    tree solve's), one on the core a quarter of that at most (its rule)."""
+    vertices moves at least 14 n-row blocks (the CG's vectors 12, the product and
+    the tree solve 2 each, 2 less in the first), one on the core about 17 of its
+    own rows, a quarter of n at most, and its indices."""
     gpu.grass_kernel_timing_enable(ctx, gpu.GRASS_KF_CG)
-    gpu.grass_embed(ctx, S, h0, r, 1, prec, 0.0, maxit)
+    gpu.grass_embed(ctx, S, h0, r, t, prec, 0.0, maxit)
     _, launches, by = gpu.grass_kernel_timing_read(ctx)
     gpu.grass_kernel_timing_enable(ctx, gpu.GRASS_KF_NONE)
-    blocks = by / (n * r * (8 if prec == gpu.GRASS_FP64 else 4)) / maxit
-    assert launches == 1 and (blocks >= 17 or blocks <= 10)
+    blocks = by / (n * r * (8 if prec == gpu.GRASS_FP64 else 4)) / (maxit * t)
+    assert launches == t and (blocks >= 14 or blocks <= 10)
     return blocks <= 10
 
 
@@ -204,3 +205,23 @@ def test_core_without_room_serves_over_all_vertices(gpu, leave_mb):
         finally:
             for S in made:
                 gpu.grass_sparsifier_destroy(S)
+
+
+@pytest.mark.parametrize("side,r,maxit,t,core", [(60, 2, 16, 1, False), (60, 2, 159, 1, False),
+                                                 (60, 2, 160, 1, True), (60, 2, 80, 2, True),
+                                                 (300, 32, 11, 1, False), (300, 32, 12, 1, True),
+                                                 (300, 32, 6, 2, True)])
+def test_core_waits_for_iterations_that_pay_its_build(gpu, side, r, maxit, t, core):
+    """The rule's sides in the iterations a call allows: 160, or 256 MB over the
+    block's bytes (23 MB here)."""
+    g = graphs.grid2d_uniform(side, side, seed=9)
+    ot = oracle.build_tree(oracle.from_graph(g))
+    add = np.flatnonzero(ot.in_tree == 0)[::97].astype(np.int64)
+    with gpu_graph(g) as (ctx, tree, _):
+        S = gpu.grass_sparsifier_create(ctx, tree)
+        try:
+            gpu.grass_sparsifier_add(ctx, S, dev(add))
+            h0 = dev(rng.gaussian_block(12, 3, g.n, r))
+            assert _on_core(gpu, ctx, S, g.n, h0, r, gpu.GRASS_FP64, maxit, t) == core
+        finally:
+            gpu.grass_sparsifier_destroy(S)
