@@ -225,3 +225,112 @@ def test_core_waits_for_iterations_that_pay_its_build(gpu, side, r, maxit, t, co
             assert _on_core(gpu, ctx, S, g.n, h0, r, gpu.GRASS_FP64, maxit, t) == core
         finally:
             gpu.grass_sparsifier_destroy(S)
+
+
+@pytest.mark.parametrize("r,prec", [(8, "fp64"), (16, "fp64"), (24, "fp64"), (32, "fp64"),
+                                    (16, "fp32"), (24, "fp32"), (32, "fp32")])
+@pytest.mark.parametrize("sms", [0, 4])
+def test_core_columns_in_groups(gpu, r, prec, sms):
+    """Every count of column groups a unit is worked on in, spread over the grid
+    (sms = 0: more thread groups than units) and one after the other in the
+    group that has staged the unit's lists (4 SMs: fewer)."""
+    import torch
+    g = graphs.grid3d_loguniform(22, 21, 20, seed=3)
+    og = oracle.from_graph(g)
+    ot = oracle.build_tree(og)
+    add = np.flatnonzero(ot.in_tree == 0)[::97]
+    in_s = ot.in_tree.copy()
+    in_s[add] = 1
+    h0 = rng.gaussian_block(11, 4, g.n, r)
+    ref, _ = oracle.heat(og, in_s, oracle.embed(og, ot, in_s, h0, 1, 1e-13, 3000))
+    P, dt, bound, tol, maxit = ((gpu.GRASS_FP64, torch.float64, 1e-10, 1e-13, 3000) if prec == "fp64"
+                                else (gpu.GRASS_FP32, torch.float32, 1e-3, 1e-6, 200))
+    with gpu_graph(g) as (ctx, tree, _):
+        gpu.grass_ctx_set_param(ctx, "grid_sms", sms)
+        S = gpu.grass_sparsifier_create(ctx, tree)
+        try:
+            gpu.grass_sparsifier_add(ctx, S, dev(add.astype(np.int64)))
+            heat = torch.empty(ref.shape[0], dtype=dt, device="cuda")
+            gpu.grass_embed(ctx, S, dev(h0), r, 1, P, tol, maxit, None, heat)
+            assert np.abs(host(heat).astype(np.float64) - ref).max() <= bound * ref.max()
+            assert _on_core(gpu, ctx, S, g.n, dev(h0), r, P)
+        finally:
+            gpu.grass_sparsifier_destroy(S)
+
+
+@pytest.mark.parametrize("added,core", [(126, True), (128, True), (129, True), (130, False), (200, False)])
+def test_core_rule_in_added_edges(gpu, added, core):
+    """2070 vertices: 129 added edges are the last that take the core."""
+    g = graphs.grid2d_uniform(45, 46, seed=9)
+    ot = oracle.build_tree(oracle.from_graph(g))
+    add = np.flatnonzero(ot.in_tree == 0)[:added].astype(np.int64)
+    with gpu_graph(g) as (ctx, tree, _):
+        S = gpu.grass_sparsifier_create(ctx, tree)
+        try:
+            gpu.grass_sparsifier_add(ctx, S, dev(add))
+            assert _on_core(gpu, ctx, S, g.n, dev(rng.gaussian_block(12, 3, g.n, 4)), 4, gpu.GRASS_FP64) == core
+        finally:
+            gpu.grass_sparsifier_destroy(S)
+
+
+def test_core_capped_solve_of_a_large_graph(gpu):
+    """Solves that end at their cap on the core (8 iterations): the iterate is
+    the oracle's.  Tolerance: a start block moved by 1e-15 moves the oracle's own
+    heats by 6e-12 of the largest here; rounding moves the vectors of 8
+    iterations by up to some 1e-13, a hundred times that, and 1e-8 leaves a
+    factor of 16 (one iteration more changes 0.8)."""
+    import torch
+    g = graphs.grid2d_uniform(725, 724, seed=21)
+    og = oracle.from_graph(g)
+    ot = oracle.build_tree(og)
+    add = np.flatnonzero(ot.in_tree == 0)[::17]
+    in_s = ot.in_tree.copy()
+    in_s[add] = 1
+    h0 = rng.gaussian_block(11, 5, g.n, 8)
+    ref, _ = oracle.heat(og, in_s, oracle.embed(og, ot, in_s, h0, 1, 1e-13, 8))
+    with gpu_graph(g) as (ctx, tree, _):
+        S = gpu.grass_sparsifier_create(ctx, tree)
+        try:
+            gpu.grass_sparsifier_add(ctx, S, dev(add.astype(np.int64)))
+            heat = torch.empty(ref.shape[0], dtype=torch.float64, device="cuda")
+            gpu.grass_embed(ctx, S, dev(h0), 8, 1, gpu.GRASS_FP64, 1e-13, 8, None, heat)
+            assert np.abs(host(heat) - ref).max() <= 1e-8 * ref.max()
+            assert _on_core(gpu, ctx, S, g.n, dev(h0), 8, gpu.GRASS_FP64, 8)
+        finally:
+            gpu.grass_sparsifier_destroy(S)
+
+
+def test_core_above_a_quarter_is_not_used(gpu):
+    """A binary tree of 262 leaves whose 522 branches are chains of three
+    vertices, the leaves joined in pairs by 131 added edges: ends and branchings
+    are a quarter of the 2096 vertices less one, the cuts between units lie on
+    chains and add to them."""
+    import torch
+    n, k = 2096, 131
+    heap = np.arange(1, 523)
+    first = 523 + 3 * (heap - 1)                       # the chain above heap vertex h
+    par = np.zeros(n, dtype=np.int64)
+    par[heap], par[first], par[first + 1], par[first + 2] = first + 2, (heap - 1) // 2, first, first + 1
+    par[2089:] = np.arange(2088, 2095)                 # the rest on one more chain
+    i, leaves = np.arange(1, n), np.arange(261, 523)
+    u, v = np.concatenate([par[1:], leaves[:k], [0]]), np.concatenate([i, leaves[k:], [n - 1]])
+    w = np.concatenate([10.0 + rng.uniform(3, 1, n - 1), 1.0 + rng.uniform(3, 2, k + 1)])
+    g = graphs.Graph("leaves", n, *graphs.csr_from_edges(n, u, v, w, 1e-3))
+    og = oracle.from_graph(g)
+    ot = oracle.build_tree(og)
+    in_s = ot.in_tree.copy()
+    add = np.flatnonzero((ot.in_tree == 0) & (og.eu >= 261))
+    in_s[add] = 1                                      # one edge stays outside S
+    h0 = rng.gaussian_block(12, 3, n, 4)
+    ref, off = oracle.heat(og, in_s, oracle.embed(og, ot, in_s, h0, 1, 1e-13, 2000))
+    assert add.size == k and off.size == 1 and 4 * (_core_at_least(g, ot, in_s) + 1) == n
+    with gpu_graph(g) as (ctx, tree, _):
+        S = gpu.grass_sparsifier_create(ctx, tree)
+        try:
+            gpu.grass_sparsifier_add(ctx, S, dev(add.astype(np.int64)))
+            heat = torch.empty(1, dtype=torch.float64, device="cuda")
+            gpu.grass_embed(ctx, S, dev(h0), 4, 1, gpu.GRASS_FP64, 1e-13, 2000, None, heat)
+            assert np.abs(host(heat) - ref).max() <= 1e-10 * ref.max()
+            assert not _on_core(gpu, ctx, S, n, dev(h0), 4, gpu.GRASS_FP64)
+        finally:
+            gpu.grass_sparsifier_destroy(S)

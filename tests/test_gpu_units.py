@@ -128,3 +128,27 @@ def test_autotune_leaves_the_tail_of_a_tree_without_one(gpu):
             for r in (1, 8):
                 best, ms = gpu.grass_autotune(ctx, tree, r, gpu.GRASS_FP32)
                 assert best[2] == tail and best[0] in (256, 512, 1024) and ms > 0
+
+
+@pytest.mark.parametrize("kind,n", [("random", 20011), ("star", 9001), ("random", 280001)])
+@pytest.mark.parametrize("r,prec", [(16, "fp64"), (32, "fp64"), (32, "fp32")])
+def test_unit_solve_in_column_groups(gpu, kind, n, r, prec):
+    """More than one column group a unit, with units in number below and (on 4
+    SMs, or from 272,384 vertices on) above the grid's thread groups."""
+    import torch
+    g = _graph(kind, n, 9)
+    rho = n // 3
+    og = oracle.from_graph(g)
+    ot = oracle.build_tree(og, rho)
+    P, dt, tol = ((gpu.GRASS_FP64, torch.float64, 1e-10) if prec == "fp64"
+                  else (gpu.GRASS_FP32, torch.float32, 1e-4))
+    B = rng.gaussian_block(5, 8, n, r).astype(np.float32).astype(np.float64)
+    ref = oracle.tree_solve(og, ot, B, og.D)
+    with gpu_graph(g, rho) as (ctx, tree, _):
+        Bd = dev(B, dt)
+        X, Y = torch.full_like(Bd, float("nan")), torch.full_like(Bd, float("nan"))
+        gpu.grass_tree_solve(ctx, tree, 1, r, P, Bd, X)
+        assert np.abs(host(X).astype(np.float64) - ref).max() <= tol * np.abs(ref).max()
+        gpu.grass_ctx_set_param(ctx, "grid_sms", 4)
+        gpu.grass_tree_solve(ctx, tree, 1, r, P, Bd, Y)
+        assert torch.equal(X, Y)
