@@ -193,6 +193,7 @@ __device__ __forceinline__ bool cg_dev(const CGArgs<T> &g, const TreeKArgs<T> &t
                                        unsigned int &epoch, T *ys, bool preset = false,
                                        CoreScalars *cs = nullptr, const T *dv = nullptr) {
     static_assert(!EU || R == 1, "the scan-form solve handles one column");
+    static_assert(!CORE || R > 1, "one column takes the scan form");
     constexpr int TPR = Lay<R>::TPR, EPT = Lay<R>::EPT;
     __shared__ double s_red[32][32];
     __shared__ double s_rz[32], s_rr[32], s_yy[32], s_pq[32], s_new[32], s_al[32];
@@ -501,12 +502,6 @@ __device__ __forceinline__ bool cg_dev(const CGArgs<T> &g, const TreeKArgs<T> &t
                     st_chunk(g.Rv + i0, cnt, rr);
                 }
                 st_chunk(g.Z + i0, cnt, rr);
-                if constexpr (CORE) {
-                    T d[W];
-                    ld_chunk(dv + i0, cnt, d);
-#pragma unroll
-                    for (int w = 0; w < W; ++w) rr[w] += (T)cs->r[0] * d[w];
-                }
 #pragma unroll
                 for (int w = 0; w < W; ++w) {
                     if (w >= cnt) break;

@@ -523,7 +523,8 @@ static void core_T(const CoreCall &c) {
 
 template <int R>
 static void core_R(const CoreCall &c) {
-    if (c.prec == GRASS_FP64) core_T<double, R>(c);
+    if constexpr (R == 1) fail(GRASS_ERR_INVALID, "the core takes more than one column");
+    else if (c.prec == GRASS_FP64) core_T<double, R>(c);
     else core_T<float, R>(c);
 }
 
