@@ -880,6 +880,23 @@ __device__ inline bool grid_sync(unsigned int *bar, long long budget, int *err,
     return s_ok != 0;
 }
 
+// Order of two vertices in a contraction round, another one every round: by a
+// hash (the published 32-bit finaliser of MurmurHash3, A. Appleby) of the
+// vertex and the round, then by the vertex.
+__device__ inline uint32_t fmix32(uint32_t h) {
+    h ^= h >> 16;
+    h *= 0x85ebca6bu;
+    h ^= h >> 13;
+    h *= 0xc2b2ae35u;
+    h ^= h >> 16;
+    return h;
+}
+__device__ inline bool prio_gt(uint32_t a, uint32_t b, uint32_t round) {
+    const uint32_t ha = fmix32(a * 0x9E3779B1u + round * 0x7F4A7C15u);
+    const uint32_t hb = fmix32(b * 0x9E3779B1u + round * 0x7F4A7C15u);
+    return ha != hb ? ha > hb : a > b;
+}
+
 // block-wide max of a non-negative double, one atomicMax on its bit pattern
 __device__ inline void block_atomic_max(unsigned long long *maxbits, double v) {
     __shared__ double sm[32];

@@ -25,21 +25,6 @@
 
 namespace grass {
 
-__device__ inline uint32_t fmix32(uint32_t h) {
-    h ^= h >> 16;
-    h *= 0x85ebca6bu;
-    h ^= h >> 13;
-    h *= 0xc2b2ae35u;
-    h ^= h >> 16;
-    return h;
-}
-
-__device__ inline bool prio_gt(int32_t a, int32_t b, int round) {
-    uint32_t ha = fmix32((uint32_t)a * 0x9E3779B1u + (uint32_t)round * 0x7F4A7C15u);
-    uint32_t hb = fmix32((uint32_t)b * 0x9E3779B1u + (uint32_t)round * 0x7F4A7C15u);
-    return ha != hb ? ha > hb : a > b;
-}
-
 // ---------------------------------------------------------------- tree adjacency
 
 __global__ void k_tcount(int64_t n, const int32_t *adj_ptr, const int32_t *adj_eid,

@@ -78,19 +78,6 @@ __global__ void k_un_cross(int64_t n, int B, const int32_t *parent, uint8_t *pin
     else if (p / B != i / B) pin[p] = 1;
 }
 
-__device__ inline uint32_t un_hash(uint32_t h) {
-    h ^= h >> 16;
-    h *= 0x85ebca6bu;
-    h ^= h >> 13;
-    h *= 0xc2b2ae35u;
-    return h ^ h >> 16;
-}
-__device__ inline bool un_prio_gt(uint32_t a, uint32_t b, uint32_t round) {
-    const uint32_t ha = un_hash(a * 0x9E3779B1u + round * 0x7F4A7C15u);
-    const uint32_t hb = un_hash(b * 0x9E3779B1u + round * 0x7F4A7C15u);
-    return ha != hb ? ha > hb : a > b;
-}
-
 // exclusive block scan of one int per thread; *total = the block's sum
 __device__ inline int un_scan(int v, int *total) {
     __shared__ int ws[32];
@@ -207,8 +194,8 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_unit_build(UnitBuildArgs a
             if (!take) {
                 const int p = par[i], c = xch[i];
                 take = cls[c] != 1;
-                if (take && p < size && cls[p] == 2) take = un_prio_gt(base + i, base + p, rounds);
-                if (take && cls[c] == 2) take = un_prio_gt(base + i, base + c, rounds);
+                if (take && p < size && cls[p] == 2) take = prio_gt(base + i, base + p, rounds);
+                if (take && cls[c] == 2) take = prio_gt(base + i, base + c, rounds);
             }
             if (take) {
                 er[i] = (uint8_t)rounds;
@@ -232,8 +219,8 @@ __global__ void __launch_bounds__(kBuildThreads, 1) k_unit_build(UnitBuildArgs a
         for (int i = tid; i < size; i += nt) {
             if (cls[i] != 2 || !out[i]) continue;
             const int p = par[i], c = xch[i];
-            if (p < size && cls[p] == 2 && out[p] && !un_prio_gt(base + i, base + p, rounds)) continue;
-            if (cls[c] == 2 && out[c] && !un_prio_gt(base + i, base + c, rounds)) continue;
+            if (p < size && cls[p] == 2 && out[p] && !prio_gt(base + i, base + p, rounds)) continue;
+            if (cls[c] == 2 && out[c] && !prio_gt(base + i, base + c, rounds)) continue;
             er[i] = (uint8_t)rounds;
             n1[i] = (uint16_t)p;
             n2[i] = (uint16_t)c;
