@@ -126,21 +126,29 @@ __global__ void k_co_sort(int64_t nnz, int64_t n1, const int32_t *parent, const 
 // then below n / 4 and its build (about 1 ms at a million vertices, every
 // change of S) is a fraction of one solve.
 // And the iterations a caller allows on S have to pay the build, which its
-// first solve waits for: 160 of them, or fewer where a block is large (their
-// number times the block's bytes 256 MB: 8 iterations at 32 MB).  Measured, us,
-// CG over all vertices / on the core an iteration, the build, iterations that
-// pay it, with n / 17 added edges:  90,000 vertices 2 FP32 columns (0.7 MB) 49 /
-// 45, 565, 147;  90,000, 16 FP32 (5.8 MB) 76 / 65, 590, 55;  250,000, 4 FP64
-// (8 MB) 102 / 65, 636, 18;  250,000, 16 FP32 (16 MB) 111 / 73, 598, 17;
-// 1M, 4 FP64 (32 MB) 328 / 92, 965, 5;  1M, 16 FP32 (64 MB) 337 / 101, 960, 4;
-// with n / 200: 40, 25, 11, 11, 4 and 3 iterations.  The rule looks at the call
-// alone: a sparsifier solved again and again by the same short call gets the
-// same form, and the same bits, every time.
-static bool core_wanted(const grass_sparsifier_s *S, int r, size_t es, int64_t its) {
+// first solve waits for: 160 of them in FP32 and 64 in FP64, or fewer where a
+// block is large (their number times the block's bytes 256 MB, in FP64 128 MB).
+// Measured, us: an iteration over all vertices / on the core, the build with
+// n / 17 added edges, the iterations that pay it (with n / 200 added edges):
+//   90,000 vertices  2 FP32 columns (0.7 MB)  49 / 45   565  147 (40)
+//                   16 FP32 (5.8 MB)          76 / 65   590   55 (25)
+//                    2 FP64 (1.4 MB)          65 / 55   586   59 (23)
+//                   16 FP64 (11.5 MB)        122 / 66   556   11 (7)
+//   250,000         16 FP32 (16 MB)          111 / 73   598   17 (11)
+//                    4 FP64 (8 MB)           102 / 65   636   18 (11)
+//   1M               2 FP32 (8 MB)           104 / 56   962   21 (13)
+//                   16 FP32 (64 MB)          337 / 101  960    4 (3)
+//                    2 FP64 (16 MB)          198 / 77   966    9 (6)
+//                   16 FP64 (128 MB)         955 / 223  974    2 (1)
+// The rule looks at the call alone: a sparsifier solved again and again by the
+// same short call gets the same form, and the same bits, every time.
+static bool core_wanted(const grass_sparsifier_s *S, int r, grass_prec prec, int64_t its) {
     const grass_tree_s *T = S->tree;
     const int64_t n = T->g.n, added = S->n_edges - (n - 1);
+    const bool f64 = prec == GRASS_FP64;
     return T->units.built && n >= 2048 && added > 0 && 16 * added <= n &&
-           (its >= 160 || (double)its * (double)n * r * es >= (double)((size_t)256 << 20));
+           (its >= (f64 ? 64 : 160) ||
+            (double)its * (double)n * r * (f64 ? 8.0 : 4.0) >= (f64 ? 128e6 : 256e6));
 }
 
 // False: S keeps the CG over all vertices.
@@ -530,7 +538,7 @@ static void core_R(const CoreCall &c) {
 
 bool core_solve(grass_ctx_t ctx, grass_sparsifier_t S, int r, grass_prec prec, const void *Y, void *X,
                 double tol, int maxit, unsigned long long *maxbits, int64_t its) {
-    if (!core_wanted(S, r, prec == GRASS_FP64 ? 8 : 4, its) || !core_build(ctx, S)) return false;
+    if (!core_wanted(S, r, prec, its) || !core_build(ctx, S)) return false;
     CoreCall c{ctx, S, prec, Y, X, tol, maxit, maxbits};
     GRASS_DISPATCH_R(r, core_R, c);
     return true;

@@ -207,13 +207,15 @@ def test_core_without_room_serves_over_all_vertices(gpu, leave_mb):
                 gpu.grass_sparsifier_destroy(S)
 
 
-@pytest.mark.parametrize("side,r,maxit,t,core", [(60, 2, 16, 1, False), (60, 2, 159, 1, False),
-                                                 (60, 2, 160, 1, True), (60, 2, 80, 2, True),
-                                                 (300, 32, 11, 1, False), (300, 32, 12, 1, True),
-                                                 (300, 32, 6, 2, True)])
-def test_core_waits_for_iterations_that_pay_its_build(gpu, side, r, maxit, t, core):
-    """The rule's sides in the iterations a call allows: 160, or 256 MB over the
-    block's bytes (23 MB here)."""
+@pytest.mark.parametrize("side,r,prec,maxit,t,core", [
+    (60, 2, "fp64", 8, 1, False), (60, 2, "fp64", 63, 1, False), (60, 2, "fp64", 64, 1, True),
+    (60, 2, "fp64", 32, 2, True), (300, 2, "fp32", 159, 1, False), (300, 2, "fp32", 160, 1, True),
+    (300, 32, "fp64", 5, 1, False), (300, 32, "fp64", 6, 1, True), (300, 32, "fp64", 3, 2, True),
+    (300, 32, "fp32", 22, 1, False), (300, 32, "fp32", 23, 1, True)])
+def test_core_waits_for_iterations_that_pay_its_build(gpu, side, r, prec, maxit, t, core):
+    """The rule's sides in the iterations a call allows: 64 in FP64 and 160 in
+    FP32, or 128 and 256 MB over the block's bytes (23 and 11.5 MB here)."""
+    P = gpu.GRASS_FP64 if prec == "fp64" else gpu.GRASS_FP32
     g = graphs.grid2d_uniform(side, side, seed=9)
     ot = oracle.build_tree(oracle.from_graph(g))
     add = np.flatnonzero(ot.in_tree == 0)[::97].astype(np.int64)
@@ -222,7 +224,7 @@ def test_core_waits_for_iterations_that_pay_its_build(gpu, side, r, maxit, t, co
         try:
             gpu.grass_sparsifier_add(ctx, S, dev(add))
             h0 = dev(rng.gaussian_block(12, 3, g.n, r))
-            assert _on_core(gpu, ctx, S, g.n, h0, r, gpu.GRASS_FP64, maxit, t) == core
+            assert _on_core(gpu, ctx, S, g.n, h0, r, P, maxit, t) == core
         finally:
             gpu.grass_sparsifier_destroy(S)
 
