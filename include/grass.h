@@ -155,8 +155,8 @@ grass_status grass_ctx_set_wait_limit(grass_ctx_t ctx, int64_t polls, int hold_b
  *                         prefix sums: along the Euler tour for a solve on
  *                         its own, over the preorder's vertex slots inside
  *                         the inner CG and the power steps, whose vectors
- *                         are then kept in preorder); 0: the elimination
- *                         rounds
+ *                         are then kept in preorder); 0: the units or
+ *                         elimination rounds of the other solves
  *   "similarity_check"    0 (default) or 1: grass_densify filters each
  *                         round's edges with the similarity check of
  *                         grass_filter_similar (Sec. IV-D step 6)
@@ -224,12 +224,14 @@ grass_status grass_ctx_set_param(grass_ctx_t ctx, const char *name, int64_t valu
  *                    (the embedding's power steps), same bytes
  *   GRASS_KF_SPMM_S  the same over the sparsifier's adjacency (+ns with D)
  *   GRASS_KF_HEAT    m_off(8+s) + nrs + m_off s
- *   GRASS_KF_TREE    one whole tree solve:
- *                    4nrs + receivers(16+2s) + (n-1)(16+4s)
+ *   GRASS_KF_TREE    one whole tree solve: in units 2nrs + n(10+4s), in
+ *                    rounds 4nrs + receivers(16+2s) + (n-1)(16+4s)
  *   GRASS_KF_CG      one fused inner CG solve on the sparsifier: its
  *                    iterations (read back from the device) times
  *                    [tree solve + SpMV over S + 12nrs] plus 2nrs (+nrs
- *                    for max |X|, +2nrs for a preorder scatter)
+ *                    for max |X|, +2nrs for a preorder scatter); on the
+ *                    sparsifier's core those of its n1 rows, [... + 13 n1 r s],
+ *                    plus 4nrs + n(10+6s) for the way there and back
  *   GRASS_KF_PCG     one fused PCG run (grass_pcg_solve, one launch per
  *                    refinement pass): its outer iterations times
  *                    [tree solve + SpMV with A + 12ns] (tree preconditioner),
@@ -258,7 +260,7 @@ grass_status grass_kernel_timing_read(grass_ctx_t ctx, double *ms, int64_t *laun
 
 /* Validate A = L_G + D (Sec. II-A), extract its edges, build the
  * maximum-weight spanning tree (ties broken by smaller edge id, so the tree
- * is unique) and the tree's elimination schedule.  The paper's backbone is a
+ * is unique) and the tree's elimination (units or schedule).  The paper's backbone is a
  * low-stretch tree (Sec. III-B); this library uses the maximum-weight tree.
  * ground: the row rho at which L_T and L_S are made invertible (the limit of
  * the tiny diagonal on one row, Sec. III-F); 0 <= ground < n.
@@ -341,8 +343,9 @@ grass_status grass_tree_graph(grass_ctx_t ctx, grass_tree_t tree, int32_t *eu, i
 grass_status grass_tree_edges(grass_ctx_t ctx, grass_tree_t tree, uint8_t *in_tree);
 
 /* X = L_T^{-1} B grounded at rho (with_D = 0; X[rho] = 0) or
- * X = (L_T + D)^{-1} B (with_D = 1), by the tree's elimination schedule
- * (Sec. III-H: linear-time tree factorization).  B, X: device, n x r.
+ * X = (L_T + D)^{-1} B (with_D = 1), by the tree's elimination (Sec. III-H:
+ * linear-time tree factorization; a single tree of at most euler_max_n vertices
+ * in units, forests and larger trees in rounds).  B, X: device, n x r.
  * B and X may alias.  r in {1, 2, 4, 8, 16, 24, 32} (other values: INVALID). */
 grass_status grass_tree_solve(grass_ctx_t ctx, grass_tree_t tree, int with_D, int r,
                               grass_prec prec, const void *B, void *X);
@@ -355,9 +358,10 @@ grass_status grass_tree_solve(grass_ctx_t ctx, grass_tree_t tree, int with_D, in
  *   Scratch: a 256-byte array compiled into the library (grid-barrier
  * counter and wait-timeout flag), held by every GPU that loads the library
  * until the process exits.  Its size does not grow with the tree; the one
- * limit it sets is that the cooperative grid times the schedule's grid
- * barriers stays below 2^31 (far above any schedule the library builds);
- * beyond it the call returns GRASS_ERR_INVALID.
+ * limit it sets is that the cooperative grid times the solve's grid
+ * barriers stays below 2^31 (far above any that the library builds);
+ * beyond it the call returns GRASS_ERR_INVALID.  A tree that solves in units
+ * holds the vectors between its levels itself, allocated with the tree.
  *   Set-up: the first call in a CUDA context (once per device, and again
  * after the application resets the device) looks up the array's address
  * there (cudaGetSymbolAddress); make that first call before any stream

@@ -200,7 +200,7 @@ struct grass_ctx_s {
     grass::Arena build_tmp;     // the tree construction's (kept up to kKeepTmp)
     int amg_fused = 1;          // 1: the multigrid PCG runs as one cooperative kernel (amg_fused.cu)
     int64_t amg_tail_n = 0;     // its levels of at most this many vertices run in one block
-    int64_t amg_warp_n = 16384; // its levels of at most this many vertices take several lanes per row
+    int64_t amg_warp_n = 16384; // its levels of at most this many vertices take a warp per row
     int64_t amg_warp_setup_n = 16384;   // hierarchy setup: levels of at most this many
                                         // vertices use the warp forms of the long-row kernels
     // a non-blocking stream of the context's own, on which multi-kernel
@@ -572,7 +572,7 @@ struct grass_tree_s {
     grass::Arena arena;               // one allocation for most of the arrays below
     grass::GraphData g;
     grass::DBuf<uint8_t> in_tree;     // [m]
-    grass::TreeSchedule sched;         // elimination rounds (built on demand when units.built)
+    grass::TreeSchedule sched;         // elimination rounds (units.built: host sizes alone, on demand)
     grass::UnitTree units;             // unit form of the solve (one tree, with a tour)
     grass::EulerTour euler;
     grass::TreeFactor lap;            // L_T grounded at rho

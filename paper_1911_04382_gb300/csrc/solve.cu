@@ -1,7 +1,9 @@
-// solve.cu -- stand-alone tree solves X = (L_T + D)^{-1} Y (or grounded),
-// in place, by the elimination schedule of tree.cu.  One cooperative launch
-// per solve (tree_solve.cuh); devices without cooperative launch get one
-// launch per round instead.
+// solve.cu -- stand-alone tree solves X = (L_T + D)^{-1} Y (or grounded), one
+// cooperative launch each: the scan form (one grounded column, euler.cu), the
+// unit form (single trees of at most euler_max_n vertices, units.cuh; reads the
+// right-hand side where it is) or, in place, the elimination rounds of tree.cu
+// (forests and larger trees, tree_solve.cuh; one launch per round on devices
+// without cooperative launch).
 #include "tree_solve.cuh"
 
 namespace grass {

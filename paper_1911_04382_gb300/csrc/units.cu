@@ -421,7 +421,8 @@ __global__ void k_un_link(int64_t n, int B, int nu, const int4 *meta, const int3
 }
 
 // Per position of a level: how many of the previous level's exports make it
-// up, their exclusive sums (one block; a few thousand entries) and cursors.
+// up, their exclusive sums and cursors.  One block, 1,024 entries a step: a few
+// thousand in a tree's own levels, up to n / 4 for a core.
 __global__ void k_un_sptr(int n1, const int32_t *lidx, const int32_t *scnt, int32_t *sptr,
                           int32_t *cur, int32_t *pos_of) {
     int run = 0;

@@ -26,7 +26,8 @@
 // reads and block barriers (0.2-0.5 us a round, 9-11 rounds a unit), then the
 // rows' way in and out; FP64 with 8 columns and more is bound by the FP64
 // pipe (about 80M operations at 16 columns).  1M vertices, 608 units of
-// 1645, per call (the rounds form in brackets): FP32 1 column 54 us (120; the
+// 1645, per call, back to back on the same buffers (the rounds form in
+// brackets; on other buffers each call 16 FP32 columns 147): FP32 1 column 54 us (120; the
 // kernel alone 29 and 121), 4 columns 68 (156), 16 columns 131 (234), FP64
 // 1 column 85 (147), 8 columns 217 (268); 90,000 vertices FP32 41-54 (80-105).
 #pragma once
